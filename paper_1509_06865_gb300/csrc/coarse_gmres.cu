@@ -13,35 +13,51 @@
 //    (gamma5^c A = D_c - sigma gamma5^c, Eq. 2.6 with a shift), whose spectrum
 //    lies in the right half plane instead of around the origin.
 //
-// Grid: G co-resident blocks; block b owns a contiguous slice of rb coarse rows.
-// Every vector the block only ever reads or writes on its own rows (the Krylov
-// basis V_i, the raw products U_i = A s_i V_i, the right-hand side, the iterate,
-// a work vector, and when room is left the deflation vectors W, A W) lives in
-// the block's shared memory (in a per-block slice of global scratch when the
-// coarse grid is too large for that); only the vector being multiplied goes to
-// global memory (`pub`), where the matvecs of the neighbouring blocks read it.
+// Everything is kept in the D_c form (g5 = gamma5^c): gA v = g5 A v = D_c v - sigma g5 v,
+// GW_l = g5 W_l, GAW_l = g5 A W_l (signs only, so no value changes).
+//
+// Grid: G co-resident blocks; block b owns a contiguous, even-aligned slice of rb
+// coarse rows.  Every vector the block only ever reads or writes on its own rows (the
+// Krylov basis V_i, the products GU_i = gA s_i V_i, the right-hand side, the iterate,
+// a work vector, and when room is left GW and GAW) lives in the block's shared
+// memory (in a per-block slice of global scratch when the coarse grid is too large
+// for that); only the vector being multiplied goes to global memory (`pub`), where
+// the matvecs of the neighbouring blocks read it.
 //
 // One Arnoldi step, classical Gram-Schmidt with a second pass, two grid-wide
 // reductions:
-//   u     = A s_j V_j                          (matvec of pub, see below)
-//   R1:   a_l = <W_l, u>, b_i = <g5 s_i V_i, u>, f_l = <g5 s_j V_j, A W_l>
-//   t     = E^-1 a;  h1_i = b_i - sum_l F_il t_l   (F_il = <g5 s_i V_i, A W_l>)
-//   w1    = g5 (u - A W t) - sum_i h1_i s_i V_i;  pub <- w1
+//   gu    = gA s_j V_j                         (matvec of pub, see below)
+//   R1:   a_l = <GW_l, gu>, b_i = <s_i V_i, gu>, f_l = <s_j V_j, GAW_l>
+//   t     = E^-1 a;  h1_i = b_i - sum_l F_il t_l   (F_il = <s_i V_i, GAW_l>)
+//   w1    = gu - GAW t - sum_i h1_i s_i V_i;  pub <- w1
 //   R2:   h2_i = <s_i V_i, w1>, ||w1||^2  (||w2||^2 = ||w1||^2 - ||h2||^2)
 //   V_j+1 = w1 - sum_i h2_i s_i V_i  (own rows only)
 // The next matvec reads w1 from pub, complete on every block after the R2
 // barrier, and corrects it on its own rows with the stored products:
-// A s_j+1 V_j+1 = s_j+1 (A w1 - sum_i h2_i U_i).  So no block ever reads a
+// gA s_j+1 V_j+1 = s_j+1 (gA w1 - sum_i h2_i GU_i).  So no block ever reads a
 // vector that another block is still writing, with two grid barriers per step.
-// Partial sums go to a [G][slots] buffer (consecutive reductions use disjoint
-// slots); after each barrier every block adds the G partials in the same
-// order, so all blocks hold bit-identical scalars and run the Givens rotations
-// and the triangular solve redundantly.  Basis vectors stay unnormalised with
-// one scale factor each.
 //
-// The grid barrier spins on a generation counter with a clock64() budget; on
+// The matvec does not need what follows from R2, so after that barrier the block
+// splits: CG_MV threads multiply, the others gather R2, finish V_j+1 and run the
+// Givens rotations (a serial chain) beside them.
+//
+// What bounds it: latency.  At 16^3 x 32 (20480 rows, 59 MB of FP32 links, L2 resident)
+// a step of the former kernel took 48 us: 18 in a matvec whose eight lanes a row went
+// through the nine hops one after another, twice (135 rows on 128 groups); 9 in the two
+// barriers; 8 gathering partial sums that lay [block][value], a sector a value; 6 in three
+// rounds of inner products; the rest in serial scalar work.  In this form it takes 18 us
+// (a whole solve of 24 steps 1.11 -> 0.43 ms).
+//
+// Partial sums go to a [slot][G] buffer (consecutive reductions use disjoint
+// slots): after each barrier a few lanes a value read them contiguously, in the same
+// order in every block, so all blocks hold bit-identical scalars and run the Givens
+// rotations and the triangular solve redundantly.  Basis vectors stay unnormalised
+// with one scale factor each.
+//
+// The grid barrier counts arrivals and spins on the count with a clock64() budget; on
 // expiry it raises a sticky error word (the kernel then returns without further
 // waits) that the host reads at its next synchronisation (MGEIG_ETIMEOUT).
+#include <algorithm>
 #include <array>
 #include <map>
 #include <mutex>
@@ -51,11 +67,14 @@
 
 namespace mgeig {
 
-constexpr int CG_THREADS = 1024;
-constexpr int CG_GATHER = 8;                      // partial sums per lane: up to 256 blocks
+constexpr int CG_THREADS = 768;                   // 85 registers a thread: a matvec thread has 12 loads in flight
+constexpr int CG_MV = 576;                        // threads of the matvec; the others finish the step before
+constexpr int CG_POST = CG_THREADS - CG_MV;
+constexpr int CG_MAXG = 256;                      // blocks at most
 constexpr int CG_NBR_SITES = 64;                  // coarse sites of a block's staged neighbour table
 constexpr int CG_MAXM = COARSE_PERSISTENT_MAXM;   // restart length limit
 constexpr int CG_MAXK = 24;                       // deflation vectors (= max N_tv)
+static_assert(CG_MAXM <= 32, "one lane per Hessenberg row");
 // partial-sum regions of consecutive reductions never overlap
 constexpr int WS = 2 * CG_MAXK + CG_MAXM + 2;     // values of one reduction
 constexpr int OFF_S1 = 0, OFF_S2 = WS, OFF_N = 2 * WS, OFF_P = 2 * WS + 2;
@@ -64,8 +83,8 @@ constexpr int CG_SLOTS = OFF_P + CG_MAXK;
 constexpr size_t CG_SMEM_LIMIT = 227 * 1024 - 1024;
 
 struct CGState {
-    unsigned int count;   // barrier arrivals (returns to 0 after every barrier)
-    unsigned int gen;     // barrier generation
+    unsigned int count;   // barrier arrivals of the running launch (0 between launches)
+    unsigned int exits;   // blocks that have left it (0 between launches)
     int status;           // sticky: 0 ok, 1 barrier timeout, 2 breakdown
     int iters;            // accumulated Arnoldi steps of all solves
 };
@@ -79,8 +98,9 @@ template <typename R>
 struct CGArgs {
     int nagg, ntv, n;              // coarse sites, test vectors, rows = nagg * 2 ntv
     int rb;                        // rows per block (the last block may own fewer)
-    int nslice;                    // owned-row vectors per block: V (m+1), U (m+1), rhs, x, w
-    int smem_slices, smem_defl;    // 1: the slices / copies of W, A W live in shared memory
+    int nslice;                    // owned-row vectors per block: V (m+1), GU (m), rhs, x, w
+    int slices;                    // matvec threads that share a row (pair); 1: none do
+    int smem_slices, smem_defl;    // 1: the slices / copies of GW, GAW live in shared memory
     const cpx<R> *Dc;              // [9][nagg][col][row]
     const void *L16;               // 16-bit links [9][nagg][re|im][row][col] (16-bit kernels)
     const float *Ls;               // their scales [9][nagg]
@@ -89,38 +109,40 @@ struct CGArgs {
     const cpx<R> *b;               // r_c
     cpx<R> *x;                     // e (output)
     cpx<R> *pub;                   // the vector being multiplied (n)
-    cpx<R> *gslices;               // G x nslice x rb, when the slices are not in shared memory
+    cpx<R> *gslices;               // nslice vectors, block by block, when the slices are not in shared memory
     int k;                         // deflation vectors (0: none)
     const cpx<R> *W, *AW;          // k x n each
     const double2 *Einv;           // k x k, row-major
-    typename Pod2<R>::T *partial;  // [G][CG_SLOTS]
+    typename Pod2<R>::T *partial;  // [CG_SLOTS][G]
     CGState *st;
     int m, maxiter;
     double tol;
     long long timeout;
 };
 
-__device__ __forceinline__ bool grid_sync(CGState *st, unsigned int nblocks, long long timeout) {
+// Barrier number *bar of a launch: every block adds one to the count and waits for
+// G times the barrier's number.  One atomic without a reply and one 16-byte poll that
+// brings the status along (the former arrive, reset, release and status read were
+// four round trips to L2).  Returns false once the status is set.
+__device__ __forceinline__ bool grid_sync(CGState *st, unsigned int nblocks, unsigned int &bar, long long timeout) {
     __syncthreads();
     __shared__ int ok;
+    bar += nblocks;
     if (threadIdx.x == 0) {
-        volatile unsigned int *vgen = &st->gen;
-        const unsigned int g0 = *vgen;
         __threadfence();
-        const unsigned int arrived = atomicAdd(&st->count, 1u);
-        if (arrived == nblocks - 1) {
-            atomicExch(&st->count, 0u);
-            __threadfence();
-            atomicAdd(&st->gen, 1u);
-        } else {
-            const long long t0 = clock64();
-            while (*vgen == g0) {
-                if (clock64() - t0 > timeout) { atomicExch(&st->status, 1); break; }
-                __nanosleep(32);
-            }
+        atomicAdd(&st->count, 1u);
+        const long long t0 = clock64();
+        int status;
+        for (;;) {
+            int4 s;   // the words of the state in order
+            asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(s.x), "=r"(s.y), "=r"(s.z), "=r"(s.w) : "l"(st) : "memory");
+            status = s.z;
+            if (status != 0 || (int)((unsigned int)s.x - bar) >= 0) break;
+            if (clock64() - t0 > timeout) { status = 1; atomicCAS(&st->status, 0, 1); break; }
         }
         __threadfence();
-        ok = *((volatile int *)&st->status) == 0;
+        ok = status == 0;
     }
     __syncthreads();
     return ok;
@@ -137,12 +159,6 @@ __device__ __forceinline__ cpx<double> ldcg(const cpx<double> *p) {
     return cpx<double>(v.x, v.y);
 }
 
-// out[t - r0] = ((Q_c - sigma)(s v))[t] = ((gamma5^c D_c - sigma)(s v))[t] for the
-// owned rows t in [r0, r1), v = the published vector; a group of TPR consecutive
-// threads shares one row: lane q takes the columns j = q (mod TPR) of all nine
-// hop blocks, and the group reduces with shuffles.
-constexpr int TPR = 8;
-
 // The neighbour aggregate of hop d of site `site`: from the block's staged table
 // (sites s0 .. s0 + CG_NBR_SITES - 1) when there is one, else from global memory.
 template <typename R>
@@ -150,78 +166,127 @@ __device__ __forceinline__ int hop_nbr(const CGArgs<R> &a, const int *snb, int s
     return snb ? snb[d * CG_NBR_SITES + site - s0] : __ldg(a.nbr + (size_t)d * a.nagg + site);
 }
 
-template <typename R>
-__device__ __forceinline__ void qmatvec(const CGArgs<R> &a, const cpx<R> *v, R s, cpx<R> *out, int r0, int r1,
-                                        const int *snb, int s0) {
-    const int n2 = 2 * a.ntv;
-    const int grp = threadIdx.x / TPR, q = threadIdx.x % TPR, ngrp = blockDim.x / TPR;
-    for (int tb = r0; tb < r1; tb += ngrp) {
-        const int t = tb + grp;
-        cpx<R> acc0, acc1;
-        if (t < r1) {
-            const int site = t / n2, row = t % n2;
-            if constexpr (sizeof(R) == 4) {
-                // n2 <= 2 * CG_MAXK = 48: a lane's (at most 6) columns of one block are
-                // loaded before they are used, so their L2 latencies overlap
-                constexpr int U = (2 * CG_MAXK + TPR - 1) / TPR;
-                for (int d = 0; d < 9; ++d) {
-                    const int nb = hop_nbr(a, snb, s0, d, site);
-                    const cpx<R> *blk = a.Dc + ((size_t)d * a.nagg + site) * n2 * n2 + row;
-                    const cpx<R> *xb = v + (size_t)nb * n2;
-                    cpx<R> bv[U], xv[U];
+// The sums over the columns of all nine hop blocks, (D_c v)[row], for the owned rows.
+// The columns of a row are cut into a.slices contiguous parts, one thread each
+// (a.slices > 1: the parts go to part[slice][row], else the sum to out), so that a
+// whole matvec is one run of independent loads per thread.  Consecutive threads take
+// consecutive row pairs (FP32) or rows (FP64) of one column: every load of a thread is
+// 16 bytes and a warp's loads are consecutive.  tid < CG_MV.
+__device__ __forceinline__ void qmatvec_part(const CGArgs<float> &a, const cpx<float> *v, cpx<float> *part,
+                                             cpx<float> *out, int r0, int nr, const int *snb, int s0, int tid) {
+    constexpr int U = 4;   // column pairs in flight
+    const int ntv = a.ntv, n2 = 2 * ntv, np = nr >> 1, CP = 9 * ntv, S = a.slices;
+    const int sl = S > 1 ? tid / np : 0;
+    if (sl >= S) return;
+    const int q0 = sl * CP / S, q1 = (sl + 1) * CP / S;
+    const float4 *D4 = reinterpret_cast<const float4 *>(a.Dc), *v4 = reinterpret_cast<const float4 *>(v);
+    const size_t next_hop = (size_t)(a.nagg - 1) * n2 * ntv;   // from a block's end to the next hop's block
+    for (int p = S > 1 ? tid - sl * np : tid; p < np; p += S > 1 ? np : CG_MV) {
+        const int row = r0 + 2 * p, site = row / n2, rin = row - site * n2;
+        int d = q0 / ntv, jp = q0 - d * ntv;
+        const float4 *pb = D4 + (((size_t)d * a.nagg + site) * n2 + 2 * jp) * ntv + (rin >> 1);
+        const float4 *px = v4 + (size_t)hop_nbr(a, snb, s0, d, site) * ntv + jp;
+        cpx<float> t0, t1;
+        for (int q = q0; q < q1; q += U) {
+            float4 b0[U], b1[U], x[U];
 #pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int j = q + u * TPR;
-                        if (j < n2) { bv[u] = blk[(size_t)j * n2]; xv[u] = ldcg(xb + j); }
+            for (int u = 0; u < U; ++u) {
+                if (q + u < q1) {
+                    b0[u] = __ldcg(pb);
+                    b1[u] = __ldcg(pb + ntv);
+                    x[u] = __ldcg(px);
+                    pb += n2;
+                    ++px;
+                    if (++jp == ntv && ++d < 9) {
+                        jp = 0;
+                        pb += next_hop;
+                        px = v4 + (size_t)hop_nbr(a, snb, s0, d, site) * ntv;
                     }
-#pragma unroll
-                    for (int u = 0; u < U; ++u)
-                        if (q + u * TPR < n2) cmac((u & 1) ? acc1 : acc0, bv[u], xv[u]);
-                }
-            } else {
-#pragma unroll 3
-                for (int d = 0; d < 9; ++d) {
-                    const int nb = hop_nbr(a, snb, s0, d, site);
-                    const cpx<R> *blk = a.Dc + ((size_t)d * a.nagg + site) * n2 * n2 + row;
-                    const cpx<R> *xb = v + (size_t)nb * n2;
-                    int j = q;
-                    for (; j + TPR < n2; j += 2 * TPR) {
-                        cmac(acc0, blk[(size_t)j * n2], ldcg(xb + j));
-                        cmac(acc1, blk[(size_t)(j + TPR) * n2], ldcg(xb + j + TPR));
-                    }
-                    if (j < n2) cmac(acc0, blk[(size_t)j * n2], ldcg(xb + j));
+                } else {
+                    b0[u] = b1[u] = x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                cmac(t0, cpx<float>(b0[u].x, b0[u].y), cpx<float>(x[u].x, x[u].y));
+                cmac(t1, cpx<float>(b0[u].z, b0[u].w), cpx<float>(x[u].x, x[u].y));
+                cmac(t0, cpx<float>(b1[u].x, b1[u].y), cpx<float>(x[u].z, x[u].w));
+                cmac(t1, cpx<float>(b1[u].z, b1[u].w), cpx<float>(x[u].z, x[u].w));
+            }
         }
-        cpx<R> acc = acc0 + acc1;
-        for (int o = 1; o < TPR; o <<= 1) {
-            acc.re += __shfl_xor_sync(0xffffffffu, acc.re, o);
-            acc.im += __shfl_xor_sync(0xffffffffu, acc.im, o);
-        }
-        if (t < r1 && q == 0) {
-            if ((t % n2) >= a.ntv) acc = -acc;
-            out[t - r0] = s * acc - (a.sigma * s) * ldcg(v + t);
-        }
+        float4 *dst = reinterpret_cast<float4 *>(S > 1 ? part + (size_t)sl * nr : out) + p;
+        *dst = make_float4(t0.re, t0.im, t1.re, t1.im);
     }
 }
 
-// The same product with 16-bit links (FP32 vectors and arithmetic): lane q takes
-// the column pairs p = q (mod TPR) of the real and imaginary planes, and every
-// hop block's sum is multiplied by the block's scale.
+__device__ __forceinline__ void qmatvec_part(const CGArgs<double> &a, const cpx<double> *v, cpx<double> *part,
+                                             cpx<double> *out, int r0, int nr, const int *snb, int s0, int tid) {
+    constexpr int U = 2;
+    const int ntv = a.ntv, n2 = 2 * ntv, CP = 9 * ntv, S = a.slices;
+    const int sl = S > 1 ? tid / nr : 0;
+    if (sl >= S) return;
+    const int q0 = sl * CP / S, q1 = (sl + 1) * CP / S;
+    const double2 *D2 = reinterpret_cast<const double2 *>(a.Dc), *v2 = reinterpret_cast<const double2 *>(v);
+    const size_t next_hop = (size_t)(a.nagg - 1) * n2 * n2;
+    for (int p = S > 1 ? tid - sl * nr : tid; p < nr; p += S > 1 ? nr : CG_MV) {
+        const int row = r0 + p, site = row / n2, rin = row - site * n2;
+        int d = q0 / ntv, jp = q0 - d * ntv;
+        const double2 *pb = D2 + (((size_t)d * a.nagg + site) * n2 + 2 * jp) * n2 + rin;
+        const double2 *px = v2 + (size_t)hop_nbr(a, snb, s0, d, site) * n2 + 2 * jp;
+        cpx<double> t0, t1;
+        for (int q = q0; q < q1; q += U) {
+            double2 b0[U], b1[U], x0[U], x1[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (q + u < q1) {
+                    b0[u] = __ldcg(pb);
+                    b1[u] = __ldcg(pb + n2);
+                    x0[u] = __ldcg(px);
+                    x1[u] = __ldcg(px + 1);
+                    pb += 2 * n2;
+                    px += 2;
+                    if (++jp == ntv && ++d < 9) {
+                        jp = 0;
+                        pb += next_hop;
+                        px = v2 + (size_t)hop_nbr(a, snb, s0, d, site) * n2;
+                    }
+                } else {
+                    b0[u] = b1[u] = x0[u] = x1[u] = make_double2(0.0, 0.0);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                cmac(t0, cpx<double>(b0[u].x, b0[u].y), cpx<double>(x0[u].x, x0[u].y));
+                cmac(t1, cpx<double>(b1[u].x, b1[u].y), cpx<double>(x1[u].x, x1[u].y));
+            }
+        }
+        (S > 1 ? part + (size_t)sl * nr : out)[p] = t0 + t1;
+    }
+}
+
+// The same sums with 16-bit links (FP32 vectors and arithmetic): TPR16 lanes share a row
+// and, with a.slices > 1, one slice of the nine hops; lane q takes the column pairs
+// p = q (mod TPR16) of the real and imaginary planes, and every hop block's sum is
+// multiplied by the block's scale.
+constexpr int TPR16 = 8;
 template <typename H>
-__device__ __forceinline__ void qmatvec16(const CGArgs<float> &a, const cpx<float> *v, float s, cpx<float> *out,
-                                          int r0, int r1, const int *snb, int s0) {
+__device__ __forceinline__ void qmatvec16(const CGArgs<float> &a, const cpx<float> *v, cpx<float> *part,
+                                          cpx<float> *out, int r0, int nr, const int *snb, int s0, int tid) {
     using HP = typename H16<H>::P;
-    const int n2 = 2 * a.ntv, np = a.ntv;
-    const int grp = threadIdx.x / TPR, q = threadIdx.x % TPR, ngrp = blockDim.x / TPR;
-    constexpr int U = (CG_MAXK + TPR - 1) / TPR;   // pairs per lane (n2 / 2 <= CG_MAXK)
+    const int n2 = 2 * a.ntv, np = a.ntv, S = a.slices;
+    const int grp = tid / TPR16, q = tid % TPR16;
+    constexpr int ngrp = CG_MV / TPR16;
+    constexpr int U = (CG_MAXK + TPR16 - 1) / TPR16;   // pairs per lane (n2 / 2 <= CG_MAXK)
     const H *L = static_cast<const H *>(a.L16);
-    for (int tb = r0; tb < r1; tb += ngrp) {
-        const int t = tb + grp;
+    const int sl = S > 1 ? grp / nr : 0;
+    const int d0 = sl * 9 / S, d1 = sl < S ? (sl + 1) * 9 / S : d0;
+    for (int tb = 0; tb < nr; tb += S > 1 ? nr : ngrp) {
+        const int t = tb + (S > 1 ? grp - sl * nr : grp);
         float ar = 0.f, ai = 0.f;
-        if (t < r1) {
-            const int site = t / n2, row = t % n2;
-            for (int d = 0; d < 9; ++d) {
+        if (t < nr) {
+            const int site = (r0 + t) / n2, row = (r0 + t) - site * n2;
+#pragma unroll 1
+            for (int d = d0; d < d1; ++d) {
                 const size_t blk = (size_t)d * a.nagg + site;
                 const int nb = hop_nbr(a, snb, s0, d, site);
                 const HP *pr = reinterpret_cast<const HP *>(L + blk * 2 * n2 * n2 + (size_t)row * n2);
@@ -231,13 +296,13 @@ __device__ __forceinline__ void qmatvec16(const CGArgs<float> &a, const cpx<floa
                 float4 xv[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const int p = q + u * TPR;
+                    const int p = q + u * TPR16;
                     if (p < np) { rv[u] = pr[p]; iv[u] = pi[p]; xv[u] = __ldcg(xb + p); }
                 }
                 float dr = 0.f, di = 0.f;
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    if (q + u * TPR < np) {
+                    if (q + u * TPR16 < np) {
                         const float2 r = H16<H>::pair(rv[u]), im = H16<H>::pair(iv[u]);
                         const float4 x = xv[u];
                         dr = fmaf(r.x, x.x, dr); dr = fmaf(-im.x, x.y, dr);
@@ -251,25 +316,36 @@ __device__ __forceinline__ void qmatvec16(const CGArgs<float> &a, const cpx<floa
                 ai = fmaf(sc, di, ai);
             }
         }
-        for (int o = 1; o < TPR; o <<= 1) {
+        for (int o = 1; o < TPR16; o <<= 1) {
             ar += __shfl_xor_sync(0xffffffffu, ar, o);
             ai += __shfl_xor_sync(0xffffffffu, ai, o);
         }
-        if (t < r1 && q == 0) {
-            cpx<float> acc(ar, ai);
-            if ((t % n2) >= a.ntv) acc = -acc;
-            out[t - r0] = s * acc - (a.sigma * s) * ldcg(v + t);
-        }
+        if (t < nr && q == 0 && sl < S) (S > 1 ? part + (size_t)sl * nr : out)[t] = cpx<float>(ar, ai);
     }
 }
 
-// the product of the kernel's link format LK (0: level precision, 1: BF16, 2: FP16)
+// the sums of the kernel's link format LK (0: level precision, 1: BF16, 2: FP16)
 template <typename R, int LK>
-__device__ __forceinline__ void matvec(const CGArgs<R> &a, const cpx<R> *v, R s, cpx<R> *out, int r0, int r1,
-                                       const int *snb, int s0) {
-    if constexpr (LK == 0) qmatvec<R>(a, v, s, out, r0, r1, snb, s0);
-    else if constexpr (LK == 1) qmatvec16<__nv_bfloat16>(a, v, s, out, r0, r1, snb, s0);
-    else qmatvec16<__half>(a, v, s, out, r0, r1, snb, s0);
+__device__ __forceinline__ void matvec_part(const CGArgs<R> &a, const cpx<R> *v, cpx<R> *part, cpx<R> *out, int r0,
+                                            int nr, const int *snb, int s0, int tid) {
+    if constexpr (LK == 0) qmatvec_part(a, v, part, out, r0, nr, snb, s0, tid);
+    else if constexpr (LK == 1) qmatvec16<__nv_bfloat16>(a, v, part, out, r0, nr, snb, s0, tid);
+    else qmatvec16<__half>(a, v, part, out, r0, nr, snb, s0, tid);
+}
+
+// Lanes that share an inner product or a sum over vectors, at most.  An FP64 shuffle
+// reduction costs the FP64 pipe (2 lanes a cycle) an addition per lane and level, so
+// few lanes share one there.
+template <typename R> struct CGLanes { static constexpr int dot = 8, row = 8, batch = 20; };
+template <> struct CGLanes<double> { static constexpr int dot = 4, row = 4, batch = 8; };
+
+template <typename R>
+__device__ __forceinline__ cpx<R> group_sum(cpx<R> v, int lanes) {
+    for (int o = lanes >> 1; o > 0; o >>= 1) {
+        v.re += __shfl_xor_sync(0xffffffffu, v.re, o);
+        v.im += __shfl_xor_sync(0xffffffffu, v.im, o);
+    }
+    return v;
 }
 
 // Scalars (partial sums, Hessenberg matrix, Givens rotations, E^-1) are kept in
@@ -281,13 +357,10 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
     using P = typename Pod2<R>::T;
     auto P2 = [](R x, R y) { return P{x, y}; };
     extern __shared__ __align__(16) unsigned char cg_dyn[];
-    __shared__ P wpart[WS];                    // this block's partial sums
-    __shared__ P h[WS];                        // grid-wide sums after a gather
-    __shared__ P F[CG_MAXM * CG_MAXK];         // F_il = <g5 s_i V_i, A W_l>
-    __shared__ P h1[CG_MAXM];
-    __shared__ P h2s[CG_MAXM];                 // second-pass coefficients of the last step
-    __shared__ R nsum[CG_THREADS / 32];
-    __shared__ R nrm2s;
+    __shared__ P h[WS];                        // grid-wide sums of the first reduction (and of the single ones)
+    __shared__ P hp[CG_MAXM + 2];              // of the second: the coefficients of the second pass, ||w1||^2
+    __shared__ P F[CG_MAXM * CG_MAXK];         // F_il = <s_i V_i, GAW_l>
+    __shared__ P hc[CG_MAXM];                  // h1_i s_i
     __shared__ P Rm[(CG_MAXM + 1) * CG_MAXM];  // rotated Hessenberg, column-major
     __shared__ R cs[CG_MAXM];
     __shared__ P sn[CG_MAXM], g[CG_MAXM + 1], y[CG_MAXM];
@@ -296,200 +369,258 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
     __shared__ R bnorm, beta;
     __shared__ int stop;
     const unsigned int G = gridDim.x;
-    const int nw = CG_THREADS / 32;
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    const int tid = threadIdx.x, lane = tid & 31;
     const int rb = a.rb;
     const int r0 = min(a.n, (int)blockIdx.x * rb);
     const int r1 = min(a.n, r0 + rb);
     const int nr = r1 - r0;
     const int m = a.m, k = a.k, n2 = 2 * a.ntv;
-    P *mypart = a.partial + (size_t)blockIdx.x * CG_SLOTS;
+    P *mypart = a.partial + blockIdx.x;   // value i of this block at mypart[i * G]
+    unsigned int bar = 0;
 
-    // owned-row slices: V_0..V_m, U_0..U_m, rhs, x, w
-    cpx<R> *S = a.smem_slices ? reinterpret_cast<cpx<R> *>(cg_dyn)
-                              : a.gslices + (size_t)blockIdx.x * a.nslice * rb;
-    auto Vv = [&](int i) { return S + (size_t)i * rb; };
-    auto Uv = [&](int i) { return S + (size_t)(m + 1 + i) * rb; };
-    cpx<R> *rhs = S + (size_t)(2 * m + 2) * rb;
-    cpx<R> *xs = rhs + rb;
-    cpx<R> *ws = xs + rb;
-    cpx<R> *Dl = a.smem_defl ? reinterpret_cast<cpx<R> *>(cg_dyn) + (size_t)a.nslice * rb : nullptr;
-    auto Wv = [&](int l) -> const cpx<R> * { return Dl ? Dl + (size_t)l * rb : a.W + (size_t)l * a.n + r0; };
-    auto AWv = [&](int l) -> const cpx<R> * { return Dl ? Dl + (size_t)(k + l) * rb : a.AW + (size_t)l * a.n + r0; };
+    // owned-row slices: V_0..V_m, GU_0..GU_m-1, rhs, x, w
+    cpx<R> *S = a.smem_slices ? reinterpret_cast<cpx<R> *>(cg_dyn) : a.gslices + (size_t)a.nslice * r0;
+    const int ld = a.smem_slices ? rb : nr;
+    auto Vv = [&](int i) { return S + (size_t)i * ld; };
+    auto Uv = [&](int i) { return S + (size_t)(m + 1 + i) * ld; };
+    cpx<R> *rhs = S + (size_t)(2 * m + 1) * ld;
+    cpx<R> *xs = rhs + ld;
+    cpx<R> *ws = xs + ld;
+    cpx<R> *dyn = reinterpret_cast<cpx<R> *>(cg_dyn) + (a.smem_slices ? (size_t)a.nslice * rb : 0);
+    cpx<R> *part = dyn;   // matvec parts [slices][nr] when a.slices > 1
+    cpx<R> *Dl = a.smem_defl ? dyn + (a.slices > 1 ? (size_t)a.slices * rb : 0) : nullptr;
     auto g5 = [&](int i, cpx<R> v) { return ((r0 + i) % n2) >= a.ntv ? -v : v; };
+    // element i of GW_l and GAW_l
+    auto GW = [&](int l, int i) { return Dl ? Dl[(size_t)l * rb + i] : g5(i, a.W[(size_t)l * a.n + r0 + i]); };
+    auto GAW = [&](int l, int i) { return Dl ? Dl[(size_t)(k + l) * rb + i] : g5(i, a.AW[(size_t)l * a.n + r0 + i]); };
 
-    // the neighbour table of the block's coarse sites, staged once (the matvec's
-    // block loads then wait on one L2 round trip per hop instead of two)
+    // the neighbour table of the block's coarse sites, staged once
     __shared__ int snb[9 * CG_NBR_SITES];
     const int s0 = nr > 0 ? r0 / n2 : 0;
     const int nsites = nr > 0 ? (r1 - 1) / n2 - s0 + 1 : 0;
     const int *snb_p = nsites <= CG_NBR_SITES ? snb : nullptr;
     if (snb_p)
-        for (int e = threadIdx.x; e < 9 * nsites; e += blockDim.x) {
+        for (int e = tid; e < 9 * nsites; e += CG_THREADS) {
             const int d = e / nsites, sl = e % nsites;
             snb[d * CG_NBR_SITES + sl] = __ldg(a.nbr + (size_t)d * a.nagg + s0 + sl);
         }
-    for (int i = threadIdx.x; i < k * k; i += blockDim.x) Ei[i] = P2((R)a.Einv[i].x, (R)a.Einv[i].y);
-    if (threadIdx.x < CG_MAXK) { tc[threadIdx.x] = P2(0, 0); t0[threadIdx.x] = P2(0, 0); }
+    for (int i = tid; i < k * k; i += CG_THREADS) Ei[i] = P2((R)a.Einv[i].x, (R)a.Einv[i].y);
+    if (tid < CG_MAXK) { tc[tid] = P2(0, 0); t0[tid] = P2(0, 0); }
     if (Dl)
-        for (int e = threadIdx.x; e < k * nr; e += blockDim.x) {
+        for (int e = tid; e < k * nr; e += CG_THREADS) {
             const int l = e / nr, i = e % nr;
-            Dl[(size_t)l * rb + i] = a.W[(size_t)l * a.n + r0 + i];
-            Dl[(size_t)(k + l) * rb + i] = a.AW[(size_t)l * a.n + r0 + i];
+            Dl[(size_t)l * rb + i] = g5(i, a.W[(size_t)l * a.n + r0 + i]);
+            Dl[(size_t)(k + l) * rb + i] = g5(i, a.AW[(size_t)l * a.n + r0 + i]);
         }
-    __syncthreads();
 
-    // wpart[i] = sc_i <X_i, u> over the owned rows, i < cnt: warp i takes value i,
-    // its lanes stride over the rows
-    auto dots = [&](int cnt, int base, auto vec, auto sc, const cpx<R> *u, bool g5x) {
-        for (int i = wp; i < cnt; i += nw) {
-            const cpx<R> *xi = vec(i);
-            R sr = 0, si = 0;
-            for (int t = lane; t < nr; t += 32) {
-                cpx<R> p = xi[t], q = u[t];
-                if (g5x) p = g5(t, p);
-                sr += p.re * q.re + p.im * q.im;
-                si += p.re * q.im - p.im * q.re;
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                sr += __shfl_xor_sync(0xffffffffu, sr, o);
-                si += __shfl_xor_sync(0xffffffffu, si, o);
-            }
-            if (lane == 0) wpart[base + i] = P2(sr * sc(i), si * sc(i));
+    // lanes per inner product (a long slice in global memory wants whole warps), per row
+    const int ldot = nr > 512 ? 32 : CGLanes<R>::dot;
+    auto row_lanes = [&](int threads) {
+        int l = 1;
+        while (l < CGLanes<R>::row && 2 * l * nr <= threads) l *= 2;
+        return l;
+    };
+    const int lrow = row_lanes(CG_THREADS), lpost = row_lanes(CG_POST);
+
+    // partial slot off + i <- val(i, t) summed over the owned rows t, i < cnt
+    auto dots = [&](int off, int cnt, auto val, auto sc) {
+        const int ngrp = CG_THREADS / ldot, q = tid & (ldot - 1);
+        for (int ib = 0; ib < cnt; ib += ngrp) {
+            const int i = ib + tid / ldot;
+            cpx<R> acc;
+            if (i < cnt) val(i, q, ldot, acc);
+            acc = group_sum(acc, ldot);
+            if (i < cnt && q == 0) mypart[(size_t)(off + i) * G] = P2(acc.re * sc(i), acc.im * sc(i));
         }
     };
-    // wpart[slot] = ||v||^2 over the owned rows
-    auto norm_part = [&](const cpx<R> *v, int slot) {
-        R acc = 0;
-        for (int t = threadIdx.x; t < nr; t += blockDim.x) {
-            cpx<R> q = v[t];
-            acc += q.re * q.re + q.im * q.im;
-        }
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) nsum[wp] = acc;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            R s2 = 0;
-            for (int w = 0; w < nw; ++w) s2 += nsum[w];
-            wpart[slot] = P2(s2, 0);
+    // acc += sum of conj(X[t]) Y[t] over the rows t = q, q + step, ...
+    auto dot_rows = [&](const cpx<R> *X, const cpx<R> *Y, int q, int step, cpx<R> &acc) {
+        for (int t = q; t < nr; t += step) cmac_conj(acc, X[t], Y[t]);
+    };
+    auto dot_gw = [&](int l, const cpx<R> *Y, int q, int step, cpx<R> &acc) {
+        if (Dl) dot_rows(Dl + (size_t)l * rb, Y, q, step, acc);
+        else for (int t = q; t < nr; t += step) cmac_conj(acc, GW(l, t), Y[t]);
+    };
+    // dst[i] = sum of value off + i over the blocks, i < cnt, by the threads [first, first + threads)
+    auto gather = [&](int off, int cnt, P *dst, int t, int threads) {
+        constexpr int L = CGLanes<R>::dot, B = CGLanes<R>::batch;
+        const int ngrp = threads / L, q = t % L;
+        for (int ib = 0; ib < cnt; ib += ngrp) {
+            const int i = ib + t / L;
+            const P *src = a.partial + (size_t)(off + i) * G;
+            cpx<R> acc;
+            if (i < cnt)
+                for (unsigned int b0 = 0; b0 < G; b0 += L * B) {
+                    P pv[B];   // loaded before they are added, so that the L2 latencies overlap
+#pragma unroll
+                    for (int u = 0; u < B; ++u) {
+                        const unsigned int b = b0 + q + L * u;
+                        pv[u] = b < G ? __ldcg(src + b) : P{0, 0};
+                    }
+#pragma unroll
+                    for (int u = 0; u < B; ++u) { acc.re += pv[u].x; acc.im += pv[u].y; }
+                }
+            acc = group_sum(acc, L);
+            if (i < cnt && q == 0) dst[i] = P2(acc.re, acc.im);
         }
     };
-    // publish wpart[0..cnt) to this block's partial slots, barrier, h = grid sums
+    // the partial sums of the block are in their slots: barrier, h = grid sums
     auto reduce = [&](int off, int cnt) -> bool {
-        __syncthreads();
-        for (int i = threadIdx.x; i < cnt; i += blockDim.x) mypart[off + i] = wpart[i];
-        if (!grid_sync(a.st, G, a.timeout)) return false;
-        for (int i = wp; i < cnt; i += nw) {
-            // all of a lane's partials are loaded before they are added (G <= 32 *
-            // CG_GATHER), so their L2 latencies overlap; the order of the sums is
-            // the same in every block
-            P pv[CG_GATHER];
-#pragma unroll
-            for (int u = 0; u < CG_GATHER; ++u) {
-                const unsigned int q = lane + 32u * u;
-                pv[u] = q < G ? __ldcg(a.partial + (size_t)q * CG_SLOTS + off + i) : P{0, 0};
-            }
-            R sr = 0, si = 0;
-#pragma unroll
-            for (int u = 0; u < CG_GATHER; ++u) { sr += pv[u].x; si += pv[u].y; }
-            for (int o = 16; o > 0; o >>= 1) {
-                sr += __shfl_xor_sync(0xffffffffu, sr, o);
-                si += __shfl_xor_sync(0xffffffffu, si, o);
-            }
-            if (lane == 0) h[i] = P2(sr, si);
-        }
+        if (!grid_sync(a.st, G, bar, a.timeout)) return false;
+        gather(off, cnt, h, tid, CG_THREADS);
         __syncthreads();
         return true;
     };
-    // u[i] = f(i, u[i], sum_l coef_l X_l[i]) on the owned rows; TPR lanes share a row
-    auto combine = [&](int cnt, auto vec, auto coef, cpx<R> *u, auto f) {
-        const int grp = threadIdx.x / TPR, q = threadIdx.x % TPR, ngrp = blockDim.x / TPR;
+    // f(i, s) with s = sum of term(l, i), l < cnt, once per owned row i, by `lanes` threads a row
+    auto rows = [&](int t, int threads, int lanes, int cnt, auto term, auto f) {
+        const int ngrp = threads / lanes, q = t & (lanes - 1);
         for (int ib = 0; ib < nr; ib += ngrp) {
-            const int i = ib + grp;
-            cpx<R> acc0, acc1;
-            if (i < nr) {
-                int l = q;
-                for (; l + TPR < cnt; l += 2 * TPR) {
-                    cmac(acc0, coef(l), vec(l)[i]);
-                    cmac(acc1, coef(l + TPR), vec(l + TPR)[i]);
-                }
-                if (l < cnt) cmac(acc0, coef(l), vec(l)[i]);
-            }
-            cpx<R> acc = acc0 + acc1;
-            for (int o = 1; o < TPR; o <<= 1) {
-                acc.re += __shfl_xor_sync(0xffffffffu, acc.re, o);
-                acc.im += __shfl_xor_sync(0xffffffffu, acc.im, o);
-            }
-            if (i < nr && q == 0) u[i] = f(i, u[i], acc);
+            const int i = ib + t / lanes;
+            cpx<R> acc;
+            if (i < nr)
+                for (int l = q; l < cnt; l += lanes) term(l, i, acc);
+            acc = group_sum(acc, lanes);
+            if (i < nr && q == 0) f(i, acc);
+        }
+    };
+    auto C = [](P p) { return cpx<R>(p.x, p.y); };
+    // finishes out = gA (s v): the parts (or the sum) of D_c v, the shift (own = v's owned
+    // rows), minus sum_l h2_l s GU_l of the l < nu earlier products
+    auto matvec_end = [&](R s, cpx<R> *out, const cpx<R> *own, int nu) {
+        const int np = a.slices > 1 ? a.slices : 0;
+        rows(tid, CG_THREADS, lrow, np + nu,
+             [&](int l, int i, cpx<R> &acc) {
+                 if (l < np) acc = acc + s * part[(size_t)l * nr + i];
+                 else cmac(acc, -(s * C(hp[l - np])), Uv(l - np)[i]);
+             },
+             [&](int i, cpx<R> acc) {
+                 const R sg = ((r0 + i) % n2) >= a.ntv ? -a.sigma : a.sigma;
+                 if (!np) acc = acc + s * out[i];
+                 out[i] = acc - (sg * s) * own[i];
+             });
+        __syncthreads();
+    };
+    // out = gA v of the published vector whose owned rows are `own`
+    auto matvec = [&](cpx<R> *out, const cpx<R> *own) {
+        if (tid < CG_MV) matvec_part<R, LK>(a, a.pub, part, out, r0, nr, snb_p, s0, tid);
+        __syncthreads();
+        matvec_end(R(1), out, own, 0);
+    };
+    // y_i = base(i) - sum_l M(i, l) x_l (l < k), i < cnt: four lanes a row
+    auto small_mv = [&](int cnt, auto M, const P *x, auto f) {
+        for (int ib = 0; ib < cnt; ib += CG_THREADS / 4) {
+            const int i = ib + tid / 4;
+            cpx<R> acc;
+            if (i < cnt)
+                for (int l = tid & 3; l < k; l += 4) cmac(acc, C(M(i, l)), C(x[l]));
+            acc = group_sum(acc, 4);
+            if (i < cnt && (tid & 3) == 0) f(i, acc);
         }
         __syncthreads();
     };
-    // u[i] = f(i, u[i], sum_l coef1_l X1_l[i], sum_l coef2_l X2_l[i]): two combines
-    // in one pass over the rows and one block barrier
-    auto combine2 = [&](int cnt1, auto vec1, auto coef1, int cnt2, auto vec2, auto coef2, cpx<R> *u, auto f) {
-        const int grp = threadIdx.x / TPR, q = threadIdx.x % TPR, ngrp = blockDim.x / TPR;
-        for (int ib = 0; ib < nr; ib += ngrp) {
-            const int i = ib + grp;
-            cpx<R> a1, a2;
-            if (i < nr) {
-                for (int l = q; l < cnt1; l += TPR) cmac(a1, coef1(l), vec1(l)[i]);
-                for (int l = q; l < cnt2; l += TPR) cmac(a2, coef2(l), vec2(l)[i]);
-            }
-            for (int o = 1; o < TPR; o <<= 1) {
-                a1.re += __shfl_xor_sync(0xffffffffu, a1.re, o);
-                a1.im += __shfl_xor_sync(0xffffffffu, a1.im, o);
-                a2.re += __shfl_xor_sync(0xffffffffu, a2.re, o);
-                a2.im += __shfl_xor_sync(0xffffffffu, a2.im, o);
-            }
-            if (i < nr && q == 0) u[i] = f(i, u[i], a1, a2);
-        }
-        __syncthreads();
-    };
-    auto publish = [&](const cpx<R> *v) {
-        for (int i = threadIdx.x; i < nr; i += blockDim.x) a.pub[r0 + i] = v[i];
+    auto einv_h = [&](P *dst) {   // dst = E^-1 h
+        small_mv(k, [&](int i, int l) { return Ei[i * k + l]; }, h, [&](int i, cpx<R> t) { dst[i] = P2(t.re, t.im); });
     };
     auto one = [](int) { return R(1); };
-    auto tcoef = [&](int l) { return cpx<R>((R)tc[l].x, (R)tc[l].y); };
-
-    // tc = E^-1 W^dag u
-    auto deflation_coeffs = [&](const cpx<R> *u) -> bool {
-        dots(k, 0, Wv, one, u, false);
+    // tc = E^-1 W^dag A x from the product gx = gA x
+    auto deflation_coeffs = [&](const cpx<R> *gx) -> bool {
+        dots(OFF_P, k, [&](int l, int q, int st, cpx<R> &acc) { dot_gw(l, gx, q, st, acc); }, one);
         if (!reduce(OFF_P, k)) return false;
-        for (int i = threadIdx.x; i < k; i += blockDim.x) {
-            R sr = 0, si = 0;
-            for (int l = 0; l < k; ++l) {
-                P e = Ei[i * k + l], d = h[l];
-                sr += e.x * d.x - e.y * d.y;
-                si += e.x * d.y + e.y * d.x;
-            }
-            tc[i] = P2(sr, si);
-        }
-        __syncthreads();
+        einv_h(tc);
         return true;
     };
-    // u <- gamma5^c (u - A W tc)
-    auto project_g5 = [&](cpx<R> *u) {
-        combine(k, AWv, tcoef, u, [&](int i, cpx<R> ui, cpx<R> s) { return g5(i, ui - s); });
+    auto gaw_t = [&](int l, int i, cpx<R> &acc) { cmac(acc, C(tc[l]), GAW(l, i)); };
+    auto publish = [&](const cpx<R> *v) {
+        for (int i = tid; i < nr; i += CG_THREADS) a.pub[r0 + i] = v[i];
+    };
+    auto norm_to = [&](const cpx<R> *v, int slot) {
+        dots(slot, 1, [&](int, int q, int st, cpx<R> &acc) { dot_rows(v, v, q, st, acc); }, one);
     };
 
     // rhs = gamma5^c Pi r_c, t0 = E^-1 W^dag r_c, x = 0.  The tolerance refers
     // to ||r_c||: when r_c lies mostly in span(W) the projected right-hand side
     // is small and needs no further reduction.
-    for (int i = threadIdx.x; i < nr; i += blockDim.x) { rhs[i] = a.b[r0 + i]; xs[i] = cpx<R>(); }
+    for (int i = tid; i < nr; i += CG_THREADS) { rhs[i] = g5(i, a.b[r0 + i]); xs[i] = cpx<R>(); }
     __syncthreads();
-    norm_part(rhs, 0);
-    if (!reduce(OFF_N, 1)) return;
-    if (threadIdx.x == 0) bnorm = sqrt(h[0].x);
+    // ||r_c||^2 and W^dag r_c in one reduction
+    dots(OFF_S1, k + 1, [&](int l, int q, int st, cpx<R> &acc) {
+        if (l < k) dot_gw(l, rhs, q, st, acc);
+        else dot_rows(rhs, rhs, q, st, acc);
+    }, one);
+    if (!reduce(OFF_S1, k + 1)) return;
+    if (tid == 0) {
+        bnorm = sqrt(h[k].x);
+        stop = !(bnorm > 0) || !isfinite(bnorm);
+    }
+    if (k > 0) einv_h(t0);
     __syncthreads();
     if (k > 0) {
-        if (!deflation_coeffs(rhs)) return;
-        for (int i = threadIdx.x; i < k; i += blockDim.x) t0[i] = tc[i];
+        rows(tid, CG_THREADS, lrow, k, [&](int l, int i, cpx<R> &acc) { cmac(acc, C(t0[l]), GAW(l, i)); },
+             [&](int i, cpx<R> s) { rhs[i] = rhs[i] - s; });
         __syncthreads();
     }
-    project_g5(rhs);
-    if (threadIdx.x == 0) stop = !(bnorm > 0) || !isfinite(bnorm);
-    __syncthreads();
     const R tol_abs = (R)a.tol * bnorm;
+
+    // what follows the second reduction of step j, by the threads that do not multiply:
+    // the coefficients, V_j+1 = w1 - sum_i h2_i s_i V_i on the owned rows (in place), and
+    // in the last warp the Hessenberg column, its rotations and the stop test
+    auto post = [&](int j) {
+        const int t = tid - CG_MV;
+        gather(OFF_S2, j + 2, hp, t, CG_POST);
+        asm volatile("bar.sync 1, %0;" ::"n"(CG_POST) : "memory");
+        cpx<R> *vn = Vv(j + 1);
+        if (t < CG_POST - 32) {
+            rows(t, CG_POST - 32, lpost, j + 1,
+                 [&](int l, int i, cpx<R> &acc) { cmac(acc, scale[l] * C(hp[l]), Vv(l)[i]); },
+                 [&](int i, cpx<R> s) { vn[i] = vn[i] - s; });
+            return;
+        }
+        P *col = Rm + j * (CG_MAXM + 1);
+        R n2s = 0;
+        if (lane <= j) {
+            const P v = hp[lane];
+            col[lane] = P2(col[lane].x + v.x, col[lane].y + v.y);
+            n2s = v.x * v.x + v.y * v.y;
+        }
+        for (int o = 16; o > 0; o >>= 1) n2s += __shfl_xor_sync(0xffffffffu, n2s, o);
+        __syncwarp();
+        if (lane == 0) {
+            n2s = hp[j + 1].x - n2s;
+            const R nrm = sqrt(n2s > 0 ? n2s : R(0));
+            P p = col[0], q;
+            for (int i = 0; i < j; ++i) {   // previous rotations
+                q = col[i + 1];
+                const P sv = sn[i];
+                const R c = cs[i];
+                col[i] = P2(c * p.x + (sv.x * q.x - sv.y * q.y), c * p.y + (sv.x * q.y + sv.y * q.x));
+                p = P2(c * q.x - (sv.x * p.x + sv.y * p.y), c * q.y - (sv.x * p.y - sv.y * p.x));
+            }
+            q = P2(nrm, 0);
+            R ap = hypot(p.x, p.y), aq = nrm;
+            R c, sr, si;
+            if (aq == 0) { c = 1; sr = 0; si = 0; }
+            else if (ap == 0) { c = 0; sr = 1; si = 0; }
+            else {
+                R tt = hypot(ap, aq);
+                c = ap / tt;
+                R ur = p.x / ap, ui = p.y / ap;          // s = (p/|p|) conj(q) / t
+                sr = (ur * q.x + ui * q.y) / tt;
+                si = (ui * q.x - ur * q.y) / tt;
+            }
+            cs[j] = c;
+            sn[j] = P2(sr, si);
+            col[j] = P2(c * p.x + (sr * q.x - si * q.y), c * p.y + (sr * q.y + si * q.x));
+            col[j + 1] = P2(0, 0);
+            P gj = g[j];
+            g[j + 1] = P2(-(sr * gj.x + si * gj.y), -(sr * gj.y - si * gj.x));
+            g[j] = P2(c * gj.x, c * gj.y);
+            const R est = hypot(g[j + 1].x, g[j + 1].y);
+            if (!isfinite(nrm) || !isfinite(est)) atomicCAS(&a.st->status, 0, 2);
+            scale[j + 1] = nrm > 0 ? R(1) / nrm : R(0);
+            stop = (est <= tol_abs) || nrm == 0 || !isfinite(est);
+        }
+    };
+
     int its = 0;
     bool have_x = false;
     while (!stop && its < a.maxiter) {
@@ -497,26 +628,26 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
         // V0 = rhs - op(x)  (or rhs)
         if (have_x) {
             publish(xs);
-            if (!grid_sync(a.st, G, a.timeout)) return;       // x complete everywhere
-            matvec<R, LK>(a, a.pub, R(1), v0, r0, r1, snb_p, s0);
-            __syncthreads();
+            if (!grid_sync(a.st, G, bar, a.timeout)) return;   // x complete everywhere
+            matvec(v0, xs);
             if (k > 0) {
                 if (!deflation_coeffs(v0)) return;             // its barrier also ends the reads of pub
-            } else if (!grid_sync(a.st, G, a.timeout)) {
+            } else if (!grid_sync(a.st, G, bar, a.timeout)) {
                 return;                                        // every matvec done before pub changes
             }
-            combine(k, AWv, tcoef, v0, [&](int i, cpx<R> vi, cpx<R> s) { return rhs[i] - g5(i, vi - s); });
+            rows(tid, CG_THREADS, lrow, k, gaw_t, [&](int i, cpx<R> s) { v0[i] = rhs[i] - (v0[i] - s); });
         } else {
-            for (int i = threadIdx.x; i < nr; i += blockDim.x) v0[i] = rhs[i];
-            __syncthreads();
+            for (int i = tid; i < nr; i += CG_THREADS) v0[i] = rhs[i];
         }
+        __syncthreads();
         publish(v0);
-        norm_part(v0, 0);
+        for (int i = tid; i < nr; i += CG_THREADS) ws[i] = v0[i];
+        norm_to(v0, OFF_N);
         if (!reduce(OFF_N, 1)) return;                         // also makes V0 visible in pub
-        if (threadIdx.x == 0) {
+        if (tid == 0) {
             beta = sqrt(h[0].x);
             stop = !(beta > tol_abs) || !isfinite(beta);
-            if (!isfinite(beta)) atomicExch(&a.st->status, 2);
+            if (!isfinite(beta)) atomicCAS(&a.st->status, 0, 2);
             scale[0] = beta > 0 ? R(1) / beta : R(0);
             g[0] = P2(beta, 0);
             for (int i = 1; i <= CG_MAXM; ++i) g[i] = P2(0, 0);
@@ -526,120 +657,59 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
         const int mm = min(m, a.maxiter - its);
         int kk = 0;
         bool conv = false;
-        for (int j = 0; j < mm; ++j) {
-            cpx<R> *uj = Uv(j);
-            const cpx<R> *vj = Vv(j);
-            // U_j = A s_j V_j: the matvec of pub (= V_j before its second pass),
-            // corrected by the second-pass coefficients of the last step
-            matvec<R, LK>(a, a.pub, (R)scale[j], uj, r0, r1, snb_p, s0);
-            __syncthreads();
-            if (j > 0)
-                combine(j, Uv, [&](int i) { return cpx<R>((R)(h2s[i].x * scale[j]), (R)(h2s[i].y * scale[j])); },
-                        uj, [](int, cpx<R> ui, cpx<R> s) { return ui - s; });
-            // reduction 1: a_l = <W_l, u>, b_i = <g5 s_i V_i, u>, f_l = <g5 s_j V_j, A W_l>
-            dots(k, 0, Wv, one, uj, false);
-            dots(j + 1, k, Vv, [&](int i) { return scale[i]; }, uj, true);
-            for (int l = wp; l < k; l += nw) {
-                const cpx<R> *awl = AWv(l);
-                R sr = 0, si = 0;
-                for (int t = lane; t < nr; t += 32) {
-                    cpx<R> pv = g5(t, vj[t]), q = awl[t];
-                    sr += pv.re * q.re + pv.im * q.im;
-                    si += pv.re * q.im - pv.im * q.re;
-                }
-                for (int o = 16; o > 0; o >>= 1) {
-                    sr += __shfl_xor_sync(0xffffffffu, sr, o);
-                    si += __shfl_xor_sync(0xffffffffu, si, o);
-                }
-                if (lane == 0) wpart[k + j + 1 + l] = P2(sr * scale[j], si * scale[j]);
+        for (int j = 0;; ++j) {
+            // GU_j = gA s_j V_j: the matvec of pub (= V_j before its second pass) while the
+            // other threads finish step j - 1, then the correction by its second-pass
+            // coefficients.  When step j - 1 was the last the product is not used (a faster
+            // block may already write x to pub meanwhile)
+            cpx<R> *uj = Uv(min(j, m - 1));
+            if (tid < CG_MV) {
+                if (j < mm) matvec_part<R, LK>(a, a.pub, part, uj, r0, nr, snb_p, s0, tid);
+            } else if (j > 0) {
+                post(j - 1);
             }
+            __syncthreads();
+            kk = j;
+            if (j > 0 && stop) { conv = true; break; }
+            if (j == mm) break;
+            matvec_end((R)scale[j], uj, ws, j);
+            // reduction 1: a_l = <GW_l, gu>, b_i = <s_i V_i, gu>, f_l = <s_j V_j, GAW_l>
+            const cpx<R> *vj = Vv(j);
+            dots(OFF_S1, 2 * k + j + 1, [&](int l, int q, int st, cpx<R> &acc) {
+                if (l < k) dot_gw(l, uj, q, st, acc);
+                else if (l <= k + j) dot_rows(Vv(l - k), uj, q, st, acc);
+                else if (Dl) dot_rows(vj, Dl + (size_t)(l - j - 1) * rb, q, st, acc);
+                else for (int t = q; t < nr; t += st) cmac_conj(acc, vj[t], GAW(l - k - j - 1, t));
+            }, [&](int l) { return l < k ? R(1) : scale[l <= k + j ? l - k : j]; });
             if (!reduce(OFF_S1, 2 * k + j + 1)) return;
             // t = E^-1 a ; F row j ; h1_i = b_i - sum_l F_il t_l
-            for (int l = threadIdx.x; l < k; l += blockDim.x) F[j * CG_MAXK + l] = h[k + j + 1 + l];
-            for (int i = threadIdx.x; i < k; i += blockDim.x) {
-                R sr = 0, si = 0;
-                for (int l = 0; l < k; ++l) {
-                    P e = Ei[i * k + l], d = h[l];
-                    sr += e.x * d.x - e.y * d.y;
-                    si += e.x * d.y + e.y * d.x;
-                }
-                tc[i] = P2(sr, si);
-            }
-            __syncthreads();
-            for (int i = threadIdx.x; i <= j; i += blockDim.x) {
-                P b = h[k + i];
-                for (int l = 0; l < k; ++l) {
-                    P f = F[i * CG_MAXK + l], t = tc[l];
-                    b.x -= f.x * t.x - f.y * t.y;
-                    b.y -= f.x * t.y + f.y * t.x;
-                }
-                h1[i] = b;
-                Rm[j * (CG_MAXM + 1) + i] = b;
-            }
-            __syncthreads();
-            // w1 = g5 (u - A W t) - sum_i h1_i s_i V_i, published for the next matvec
-            combine2(k, AWv, tcoef, j + 1, Vv,
-                     [&](int i) { return cpx<R>((R)(h1[i].x * scale[i]), (R)(h1[i].y * scale[i])); }, ws,
-                     [&](int i, cpx<R>, cpx<R> s1, cpx<R> s2) { return g5(i, uj[i] - s1) - s2; });
-            publish(ws);
-            // reduction 2: h2_i = <s_i V_i, w1>, ||w1||^2
-            dots(j + 1, 0, Vv, [&](int i) { return scale[i]; }, ws, false);
-            // ||w1||^2 as one more inner product (no extra block barrier)
-            dots(1, j + 1, [&](int) -> const cpx<R> * { return ws; }, one, ws, false);
-            if (!reduce(OFF_S2, j + 2)) return;
-            if (threadIdx.x == 0) {
-                R n2s = h[j + 1].x;
-                for (int i = 0; i <= j; ++i) {
-                    P &col = Rm[j * (CG_MAXM + 1) + i];
-                    col = P2(col.x + h[i].x, col.y + h[i].y);
-                    n2s -= h[i].x * h[i].x + h[i].y * h[i].y;
-                }
-                nrm2s = n2s > 0 ? n2s : R(0);
-            }
-            for (int i = threadIdx.x; i <= j; i += blockDim.x) h2s[i] = h[i];
-            __syncthreads();
-            // V_j+1 = w1 - sum_i h2_i s_i V_i on the owned rows
+            for (int l = tid; l < k; l += CG_THREADS) F[j * CG_MAXK + l] = h[k + j + 1 + l];
+            if (k > 0) einv_h(tc);
+            small_mv(j + 1, [&](int i, int l) { return F[i * CG_MAXK + l]; }, tc, [&](int i, cpx<R> s) {
+                const cpx<R> b = C(h[k + i]) - s;
+                Rm[j * (CG_MAXM + 1) + i] = P2(b.re, b.im);
+                hc[i] = P2(b.re * scale[i], b.im * scale[i]);
+            });
+            // w1 = gu - GAW t - sum_i h1_i s_i V_i, published for the next matvec
             cpx<R> *vn = Vv(j + 1);
-            combine(j + 1, Vv, [&](int i) { return cpx<R>((R)(h2s[i].x * scale[i]), (R)(h2s[i].y * scale[i])); },
-                    vn, [&](int i, cpx<R>, cpx<R> s) { return ws[i] - s; });
-            if (threadIdx.x == 0) {
-                const R nrm = sqrt(nrm2s);
-                P *col = Rm + j * (CG_MAXM + 1);
-                col[j + 1] = P2(nrm, 0);
-                for (int i = 0; i < j; ++i) {   // previous rotations
-                    P p = col[i], q = col[i + 1], sv = sn[i];
-                    col[i] = P2(cs[i] * p.x + (sv.x * q.x - sv.y * q.y), cs[i] * p.y + (sv.x * q.y + sv.y * q.x));
-                    col[i + 1] = P2(cs[i] * q.x - (sv.x * p.x + sv.y * p.y), cs[i] * q.y - (sv.x * p.y - sv.y * p.x));
-                }
-                P p = col[j], q = col[j + 1];
-                R ap = hypot(p.x, p.y), aq = hypot(q.x, q.y);
-                R c, sr, si;
-                if (aq == 0) { c = 1; sr = 0; si = 0; }
-                else if (ap == 0) { c = 0; sr = 1; si = 0; }
-                else {
-                    R tt = hypot(ap, aq);
-                    c = ap / tt;
-                    R ur = p.x / ap, ui = p.y / ap;          // s = (p/|p|) conj(q) / t
-                    sr = (ur * q.x + ui * q.y) / tt;
-                    si = (ui * q.x - ur * q.y) / tt;
-                }
-                cs[j] = c;
-                sn[j] = P2(sr, si);
-                col[j] = P2(c * p.x + (sr * q.x - si * q.y), c * p.y + (sr * q.y + si * q.x));
-                col[j + 1] = P2(0, 0);
-                P gj = g[j];
-                g[j + 1] = P2(-(sr * gj.x + si * gj.y), -(sr * gj.y - si * gj.x));
-                g[j] = P2(c * gj.x, c * gj.y);
-                const R est = hypot(g[j + 1].x, g[j + 1].y);
-                if (!isfinite(nrm) || !isfinite(est)) atomicExch(&a.st->status, 2);
-                scale[j + 1] = nrm > 0 ? R(1) / nrm : R(0);
-                stop = (est <= tol_abs) || nrm == 0 || !isfinite(est);
-            }
+            rows(tid, CG_THREADS, lrow, k + j + 1,
+                 [&](int l, int i, cpx<R> &acc) {
+                     if (l < k) gaw_t(l, i, acc);
+                     else cmac(acc, C(hc[l - k]), Vv(l - k)[i]);
+                 },
+                 [&](int i, cpx<R> s) {
+                     const cpx<R> w = uj[i] - s;
+                     vn[i] = w;
+                     ws[i] = w;
+                     a.pub[r0 + i] = w;
+                 });
             __syncthreads();
-            kk = j + 1;
-            if (stop) { conv = true; break; }
+            // reduction 2: h2_i = <s_i V_i, w1>, ||w1||^2 (gathered in post)
+            dots(OFF_S2, j + 2, [&](int l, int q, int st, cpx<R> &acc) { dot_rows(l <= j ? Vv(l) : ws, ws, q, st, acc); },
+                 [&](int l) { return l <= j ? scale[l] : R(1); });
+            if (!grid_sync(a.st, G, bar, a.timeout)) return;
         }
-        if (threadIdx.x == 0) {   // y = R^-1 g
+        if (tid == 0) {   // y = R^-1 g
             for (int i = kk - 1; i >= 0; --i) {
                 P sacc = g[i];
                 for (int l = i + 1; l < kk; ++l) {
@@ -654,26 +724,34 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
             }
         }
         __syncthreads();
-        combine(kk, Vv, [&](int i) { return cpx<R>((R)(y[i].x * scale[i]), (R)(y[i].y * scale[i])); }, xs,
-                [](int, cpx<R> xi, cpx<R> s) { return xi + s; });
+        rows(tid, CG_THREADS, lrow, kk, [&](int l, int i, cpx<R> &acc) { cmac(acc, scale[l] * C(y[l]), Vv(l)[i]); },
+             [&](int i, cpx<R> s) { xs[i] = xs[i] + s; });
+        __syncthreads();
         have_x = true;
         its += kk;
         if (conv) break;
-        if (threadIdx.x == 0) stop = 0;
+        if (tid == 0) stop = 0;
         __syncthreads();
     }
     // e = y + W (t0 - E^-1 W^dag A y)
     if (k > 0) {
         publish(xs);
-        if (!grid_sync(a.st, G, a.timeout)) return;
-        matvec<R, LK>(a, a.pub, R(1), ws, r0, r1, snb_p, s0);
-        __syncthreads();
+        if (!grid_sync(a.st, G, bar, a.timeout)) return;
+        matvec(ws, xs);
         if (!deflation_coeffs(ws)) return;
-        combine(k, Wv, [&](int i) { return cpx<R>((R)(t0[i].x - tc[i].x), (R)(t0[i].y - tc[i].y)); }, xs,
-                [](int, cpx<R> xi, cpx<R> s) { return xi + s; });
+        rows(tid, CG_THREADS, lrow, k, [&](int l, int i, cpx<R> &acc) { cmac(acc, C(t0[l]) - C(tc[l]), GW(l, i)); },
+             [&](int i, cpx<R> s) { xs[i] = xs[i] + g5(i, s); });
+        __syncthreads();
     }
-    for (int i = threadIdx.x; i < nr; i += blockDim.x) a.x[r0 + i] = xs[i];
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&a.st->iters, its);
+    for (int i = tid; i < nr; i += CG_THREADS) a.x[r0 + i] = xs[i];
+    if (tid == 0) {
+        if (blockIdx.x == 0) atomicAdd(&a.st->iters, its);
+        // the last block to leave (none waits any more) resets the counters for the next launch
+        if (atomicAdd(&a.st->exits, 1u) == G - 1) {
+            atomicExch(&a.st->count, 0u);
+            atomicExch(&a.st->exits, 0u);
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -683,13 +761,24 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
 namespace {
 
 struct CGPlan {
-    int G, rb, nslice, m;
+    int G, rb, nslice, m, slices;
     bool smem_slices, smem_defl;
     size_t dyn_smem;          // dynamic shared memory per block
     size_t off_slices, off_partial, scratch_bytes;   // global scratch layout
 };
 
 size_t align256(size_t b) { return (b + 255) / 256 * 256; }
+
+// Bytes of a block's slices (2 restart + 5 vectors of ceil(n / G) rows, at most one block
+// per 128 rows) up to which they live in shared memory: the line that
+// mgeig_mg_cycle_dev_noalloc's scratch limit is drawn by.
+template <typename R> struct SliceBudget { static constexpr size_t bytes = CG_SMEM_LIMIT - 24912; };
+template <> struct SliceBudget<double> { static constexpr size_t bytes = CG_SMEM_LIMIT - 47504; };
+// Rows a block has at least: grids below 152 blocks of these rows use fewer blocks.
+// Measured on a two-grid cycle (SAP included): 8^3 x 16 FP32 80 blocks of 16 rows 0.37 ms,
+// 10 blocks of 128 0.47; FP64 107 blocks of 12 rows 2.20 ms, 32 of 40 2.38, 10 of 128 3.76
+template <typename R> struct MinRows { static constexpr int n = 16; };
+template <> struct MinRows<double> { static constexpr int n = 12; };
 
 // the kernel instance for the context's precision and link format
 template <typename R>
@@ -706,36 +795,52 @@ const void *kernel_for(Ctx &c) {
 }
 
 template <typename R>
-CGPlan compute_plan(Ctx &c, int k) {
+CGPlan compute_plan(Ctx &c, int k, int m) {
+    using P = typename Pod2<R>::T;
     CGPlan p;
     const int n = c.nagg * 2 * c.prm.n_tv;
-    p.m = std::min(c.prm.coarse_restart, CG_MAXM);
-    int dev_sms = 0;
-    MG_CUDA(cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, c.device));
+    const size_t elem = sizeof(cpx<R>);
     cudaFuncAttributes fa;
     const void *kern = kernel_for<R>(c);
     MG_CUDA(cudaFuncGetAttributes(&fa, kern));
-    const size_t elem = sizeof(cpx<R>);
-    int G = std::max(1, std::min((n * TPR + CG_THREADS - 1) / CG_THREADS, dev_sms));
-    if (c.prm.coarse_blocks > 0) G = std::min(G, c.prm.coarse_blocks);
-    G = std::min(G, 32 * CG_GATHER);
-    p.rb = (n + G - 1) / G;
+    int cap = std::min(c.sms, CG_MAXG);
+    if (c.prm.coarse_blocks > 0) cap = std::min(cap, c.prm.coarse_blocks);
+    // where the slices live, and the scratch the documented layout takes
+    const int g128 = std::max(1, std::min((n + 127) / 128, cap)), rows = (n + g128 - 1) / g128;
+    const int restart = std::min(c.prm.coarse_restart, CG_MAXM);
+    const size_t slice_b = (size_t)(2 * restart + 5) * rows * elem;
+    p.smem_slices = slice_b <= SliceBudget<R>::bytes;
+    // the rows of a block: even, so that a pair of FP32 rows (16 bytes of a link column)
+    // never straddles two blocks
+    auto even = [](int r) { return (r + 1) / 2 * 2; };
+    p.m = m;
+    p.nslice = 2 * m + 4;
+    const size_t room = CG_SMEM_LIMIT - fa.sharedSizeBytes;
+    if (p.smem_slices) p.rb = even((n + cap - 1) / cap < MinRows<R>::n ? MinRows<R>::n : (n + cap - 1) / cap);
+    else p.rb = even(rows);
+    p.rb = std::min(p.rb, even(n));
     p.G = (n + p.rb - 1) / p.rb;   // every block owns at least one row
-    p.nslice = 2 * (p.m + 1) + 3;
-    const size_t budget = CG_SMEM_LIMIT > fa.sharedSizeBytes ? CG_SMEM_LIMIT - fa.sharedSizeBytes : 0;
-    const size_t slice_b = (size_t)p.nslice * p.rb * elem, defl_b = (size_t)2 * k * p.rb * elem;
-    p.smem_slices = slice_b <= budget;
-    p.smem_defl = p.smem_slices && k > 0 && slice_b + defl_b <= budget;
-    p.dyn_smem = p.smem_slices ? slice_b + (p.smem_defl ? defl_b : 0) : 0;
+    size_t used = p.smem_slices ? (size_t)p.nslice * p.rb * elem : 0;
+    MG_REQUIRE(used <= room, MGEIG_ECUDA);
+    // matvec threads per row (pair), as far as their partial sums fit
+    const bool l16 = sizeof(R) == 4 && c.prm.coarse_links != MGEIG_LINKS_LEVEL;
+    const int units = l16 ? p.rb * TPR16 : sizeof(R) == 4 ? p.rb / 2 : p.rb;
+    p.slices = std::max(1, std::min(CG_MV / units, l16 ? 9 : 9 * c.prm.n_tv));
+    while (p.slices > 1 && used + (size_t)p.slices * p.rb * elem > room) --p.slices;
+    if (p.slices > 1) used += (size_t)p.slices * p.rb * elem;
+    p.smem_defl = p.smem_slices && k > 0 && used + (size_t)2 * k * p.rb * elem <= room;
+    if (p.smem_defl) used += (size_t)2 * k * p.rb * elem;
+    p.dyn_smem = used;
     // global scratch: pub | slices (when not in shared memory) | partial sums
     p.off_slices = align256((size_t)n * elem);
-    p.off_partial = p.off_slices + (p.smem_slices ? 0 : align256((size_t)p.G * slice_b));
-    p.scratch_bytes = p.off_partial + align256((size_t)p.G * CG_SLOTS * sizeof(typename Pod2<R>::T));
-    MG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)p.dyn_smem));
+    const size_t slices = p.smem_slices ? 0 : align256((size_t)((n + rows - 1) / rows) * slice_b);
+    p.off_partial = p.off_slices + slices;
+    const int gmax = std::max(p.G, (n + rows - 1) / rows);
+    p.scratch_bytes = p.off_partial + align256((size_t)gmax * CG_SLOTS * sizeof(P));
+    MG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.dyn_smem));
     int per_sm = 0;
     MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, CG_THREADS, p.dyn_smem));
-    MG_REQUIRE(per_sm >= 1 && p.G <= dev_sms * per_sm, MGEIG_ECUDA);
+    MG_REQUIRE(per_sm >= 1 && p.G <= c.sms * per_sm, MGEIG_ECUDA);
     return p;
 }
 
@@ -743,13 +848,15 @@ CGPlan compute_plan(Ctx &c, int k) {
 template <typename R>
 CGPlan make_plan(Ctx &c, int k) {
     static std::mutex mu;
-    static std::map<std::array<int, 8>, CGPlan> cache;
-    const std::array<int, 8> key{c.device, c.nagg, c.prm.n_tv, std::min(c.prm.coarse_restart, CG_MAXM), k,
+    static std::map<std::array<int, 9>, CGPlan> cache;
+    // no basis longer than the steps a solve may take
+    const int m = std::min({c.prm.coarse_restart, CG_MAXM, c.prm.coarse_maxiter});
+    const std::array<int, 9> key{c.device, c.nagg, c.prm.n_tv, std::min(c.prm.coarse_restart, CG_MAXM), m, k,
                                  (int)sizeof(R), sizeof(R) == 4 ? c.prm.coarse_links : 0, c.prm.coarse_blocks};
     std::lock_guard<std::mutex> lock(mu);
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
-    const CGPlan p = compute_plan<R>(c, k);
+    const CGPlan p = compute_plan<R>(c, k, m);
     cache.emplace(key, p);
     return p;
 }
@@ -791,7 +898,7 @@ void coarse_gmres_at(Ctx &c, double sigma, const void *rc, void *ec, void *scrat
     char *sc = static_cast<char *>(scratch);
     CGArgs<R> a;
     a.nagg = c.nagg; a.ntv = c.prm.n_tv; a.n = c.nagg * 2 * c.prm.n_tv;
-    a.rb = p.rb; a.nslice = p.nslice;
+    a.rb = p.rb; a.nslice = p.nslice; a.slices = p.slices;
     a.smem_slices = p.smem_slices; a.smem_defl = p.smem_defl;
     a.Dc = static_cast<const cpx<R> *>(c.Dc.p);
     a.L16 = c.Dc16.p;

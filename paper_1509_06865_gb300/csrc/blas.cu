@@ -1,12 +1,20 @@
 // BLAS-1 on flat complex arrays (fine spinors of one precision share one
 // layout, so element-wise operations ignore it; coarse vectors are flat).
 //
-// Reductions are deterministic two-pass trees: a fixed grid of 256-thread
-// blocks accumulates grid-stride partial sums (per thread in the array's own
-// precision, then in FP64 across the block with warp shuffles), writes one
-// partial per block, and a second kernel adds the partials in a fixed order.
-// Inner products of up to 16 vectors against one vector share one read of that
-// vector (the Arnoldi / Gram-Schmidt steps of GMRES, FGMRES and Algorithm 1).
+// Reductions are deterministic two-pass trees: a fixed grid of 256-thread blocks
+// accumulates grid-stride partial sums (per thread in the array's own precision, then
+// in FP64 across the block), writes one partial per block, and the last block to
+// finish adds the partials in a fixed order.  Inner products of many vectors against
+// one vector, and updates by many vectors, are one launch: blockIdx.y cuts the vectors
+// of an inner product into chunks that share one read of y per block (the Arnoldi /
+// Gram-Schmidt steps of GMRES, FGMRES and Algorithm 1), an update keeps y in registers.
+//
+// The FP64 pipe takes half a lane a cycle and scheduler, so a warp's FP64 addition costs
+// 64 cycles of it: the block sums exchange halves of the value list between lanes (31
+// additions for 32 values; a shuffle tree per value takes 160, which was 10 us a launch).
+// Projection (two passes of inner products and updates) at 16^3 x 32, before with a launch per
+// chunk of vectors, a second kernel for the sums and uploaded coefficients, and now: 20 FP64
+// vectors 528 us, 388 us; 32 FP32 vectors 348 us, 252 us.
 #include <algorithm>
 
 #include "ds.cuh"
@@ -16,16 +24,16 @@ namespace mgeig {
 
 constexpr int RED_THREADS = 256;
 constexpr int RED_MAXBLOCKS = 1024;
-constexpr int CHUNK = 16;   // pointer slots per launch
-// vectors per launch: 16 in FP32 (bandwidth bound, fewer passes over y); 8 in
-// FP64, where the FP64 pipe bounds the kernel and 16 accumulators cost occupancy
+constexpr int MAXVEC = MAX_ITERATED + 8;   // pointer slots per launch
+// vectors that share one read of y: 16 in FP32 (bandwidth bound); 8 in FP64, where the
+// FP64 pipe bounds the kernel and 16 accumulators cost occupancy
 template <typename R> struct Chunk { static constexpr int n = sizeof(R) == 4 ? 16 : 8; };
 
 template <typename R> struct V2;
 template <> struct V2<double> { typedef double2 T; };
 template <> struct V2<float> { typedef float2 T; };
 
-struct PtrPack { const void *p[CHUNK]; };
+struct PtrPack { const void *p[MAXVEC]; };
 
 // FP32 arrays of an even number of complex values on 16-byte boundaries are
 // processed two values per float4 access
@@ -57,33 +65,98 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// block-reduce `cnt` complex values held by every thread; thread 0 writes them
-template <int MAXV>
-__device__ __forceinline__ void block_reduce_store(double (&re)[MAXV], double (&im)[MAXV], int cnt, double2 *out,
-                                                   size_t out_stride) {
-    __shared__ double sh[RED_THREADS / 32][2 * MAXV];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+// Sums v[0..N) (N a power of two <= 32) over the warp: lane l ends with the sum of
+// value l / (32 / N).  While more than one value is left, each step hands half of them
+// to the partner lane instead of adding all of them on both sides.
+template <int N>
+__device__ __forceinline__ double warp_sum_many(double (&v)[N]) {
+    const int lane = threadIdx.x & 31;
+    int m = N;
 #pragma unroll
-    for (int k = 0; k < MAXV; ++k) {
-        if (k < cnt) {
-            double a = warp_sum(re[k]), b = warp_sum(im[k]);
-            if (lane == 0) { sh[w][2 * k] = a; sh[w][2 * k + 1] = b; }
+    for (int o = 16; o > 0; o >>= 1) {
+        if (m > 1) {
+            m >>= 1;
+            const bool up = lane & o;
+#pragma unroll
+            for (int i = 0; i < N / 2; ++i) {
+                if (i < m) {
+                    const double give = up ? v[i] : v[i + m], keep = up ? v[i + m] : v[i];
+                    v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                }
+            }
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
         }
     }
-    __syncthreads();
-    if (threadIdx.x < cnt) {
-        double a = 0, b = 0;
-        for (int i = 0; i < RED_THREADS / 32; ++i) { a += sh[i][2 * threadIdx.x]; b += sh[i][2 * threadIdx.x + 1]; }
-        out[(size_t)threadIdx.x * out_stride + blockIdx.x] = make_double2(a, b);
-    }
+    return v[0];
 }
 
+// Where the sums of a reduction go: partial[vector][RED_MAXBLOCKS], one ticket per chunk
+// (zero between launches), and the results.
+struct RedOut {
+    double2 *partial;
+    unsigned int *ticket;
+    double2 *out;
+};
+
+// v = (re, im) of N / 2 values per thread -> their sums over the grid at out[j0 ..
+// j0 + cnt): block sums to the partials, and the last block of the chunk adds those
+template <int N>
+__device__ __forceinline__ void grid_reduce(double (&v)[N], int j0, int cnt, const RedOut &r) {
+    __shared__ double sh[RED_THREADS / 32][N];
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const double mine = warp_sum_many<N>(v);
+    if (lane % (32 / N) == 0) sh[w][lane / (32 / N)] = mine;
+    __syncthreads();
+    if (threadIdx.x < 2 * cnt) {
+        double a = 0;
+        for (int i = 0; i < RED_THREADS / 32; ++i) a += sh[i][threadIdx.x];
+        const size_t slot = (size_t)(j0 + threadIdx.x / 2) * RED_MAXBLOCKS + blockIdx.x;
+        reinterpret_cast<double *>(r.partial)[2 * slot + (threadIdx.x & 1)] = a;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(r.ticket + blockIdx.y, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // a warp per value, its lanes for four groups of 32 residues mod 128, the groups in order:
+    // the order of the sums is part of the result (see the note on 16-bit links at the
+    // persistent coarse solver)
+    for (int j = w; j < cnt; j += RED_THREADS / 32) {
+        const double2 *p = r.partial + (size_t)(j0 + j) * RED_MAXBLOCKS;
+        double q[8];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            double a = 0, b = 0;
+            for (int i = lane + 32 * m; i < (int)gridDim.x; i += 128) {
+                const double2 t = __ldcg(p + i);
+                a += t.x;
+                b += t.y;
+            }
+            q[2 * m] = a;
+            q[2 * m + 1] = b;
+        }
+        const double mine = warp_sum_many<8>(q);   // lane 8 m: re of group m, lane 8 m + 4: im
+        double a = 0;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) a += __shfl_sync(0xffffffffu, mine, 8 * m + (lane & 4));
+        if (lane == 0) r.out[j0 + j].x = a;
+        if (lane == 4) r.out[j0 + j].y = a;
+    }
+    if (threadIdx.x == 0) r.ticket[blockIdx.y] = 0;
+}
+
+// <X_j, y> for the chunk j = per * blockIdx.y ..
 template <typename R>
-__global__ void __launch_bounds__(RED_THREADS) multidot_kernel(PtrPack X, int k, const void *__restrict__ yv, size_t n,
-                                                               double2 *__restrict__ partial, size_t pstride, bool vec4) {
+__global__ void __launch_bounds__(RED_THREADS, 2) multidot_kernel(PtrPack X, int k, int per, const void *__restrict__ yv,
+                                                               size_t n, RedOut out, bool vec4) {
     typedef typename V2<R>::T T;
     const T *y = static_cast<const T *>(yv);
     constexpr int C = Chunk<R>::n;
+    const int j0 = blockIdx.y * per;
+    k = min(per, k - j0);
     R ar[C], ai[C];
 #pragma unroll
     for (int j = 0; j < C; ++j) { ar[j] = 0; ai[j] = 0; }
@@ -92,10 +165,14 @@ __global__ void __launch_bounds__(RED_THREADS) multidot_kernel(PtrPack X, int k,
             const float4 *y4 = static_cast<const float4 *>(yv);
             for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n / 2; i += (size_t)gridDim.x * blockDim.x) {
                 const float4 b = y4[i];
+                float4 av[C];   // loaded before they are used
+#pragma unroll
+                for (int j = 0; j < C; ++j)
+                    if (j < k) av[j] = static_cast<const float4 *>(X.p[j0 + j])[i];
 #pragma unroll
                 for (int j = 0; j < C; ++j) {
                     if (j < k) {
-                        const float4 a = static_cast<const float4 *>(X.p[j])[i];
+                        const float4 a = av[j];
                         ar[j] = fmaf(a.x, b.x, ar[j]); ar[j] = fmaf(a.y, b.y, ar[j]);
                         ar[j] = fmaf(a.z, b.z, ar[j]); ar[j] = fmaf(a.w, b.w, ar[j]);
                         ai[j] = fmaf(a.x, b.y, ai[j]); ai[j] = fmaf(-a.y, b.x, ai[j]);
@@ -111,21 +188,20 @@ __global__ void __launch_bounds__(RED_THREADS) multidot_kernel(PtrPack X, int k,
 #pragma unroll
         for (int j = 0; j < C; ++j) {
             if (j < k) {
-                T a = static_cast<const T *>(X.p[j])[i];
+                T a = static_cast<const T *>(X.p[j0 + j])[i];
                 ar[j] = fma(a.x, b.x, ar[j]); ar[j] = fma(a.y, b.y, ar[j]);
                 ai[j] = fma(a.x, b.y, ai[j]); ai[j] = fma(-a.y, b.x, ai[j]);
             }
         }
     }
-    double re[C], im[C];
+    double v[2 * C];
 #pragma unroll
-    for (int j = 0; j < C; ++j) { re[j] = ar[j]; im[j] = ai[j]; }
-    block_reduce_store<C>(re, im, k, partial, pstride);
+    for (int j = 0; j < C; ++j) { v[2 * j] = ar[j]; v[2 * j + 1] = ai[j]; }
+    grid_reduce<2 * C>(v, j0, k, out);
 }
 
 template <typename R>
-__global__ void __launch_bounds__(RED_THREADS) norm2_kernel(const void *__restrict__ xv, size_t n,
-                                                            double2 *__restrict__ partial) {
+__global__ void __launch_bounds__(RED_THREADS) norm2_kernel(const void *__restrict__ xv, size_t n, RedOut out) {
     typedef typename V2<R>::T T;
     const T *x = static_cast<const T *>(xv);
     R acc = 0;
@@ -133,38 +209,22 @@ __global__ void __launch_bounds__(RED_THREADS) norm2_kernel(const void *__restri
         T a = x[i];
         acc = fma(a.x, a.x, acc); acc = fma(a.y, a.y, acc);
     }
-    double re[1] = {(double)acc}, im[1] = {0.0};
-    block_reduce_store<1>(re, im, 1, partial, 1);
+    double v[2] = {(double)acc, 0.0};
+    grid_reduce<2>(v, 0, 1, out);
 }
 
-__global__ void resid_norm2_kernel(const double2 *__restrict__ qv, const double2 *__restrict__ v,
-                                   const double2 *__restrict__ lam, size_t n, double2 *__restrict__ partial) {
+__global__ void __launch_bounds__(RED_THREADS) resid_norm2_kernel(const double2 *__restrict__ qv,
+                                                                  const double2 *__restrict__ w,
+                                                                  const double2 *__restrict__ lam, size_t n, RedOut out) {
     const double l = lam[0].x;
     double acc = 0;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        double2 a = qv[i], b = v[i];
+        double2 a = qv[i], b = w[i];
         double rx = fma(-l, b.x, a.x), ry = fma(-l, b.y, a.y);
         acc = fma(rx, rx, acc); acc = fma(ry, ry, acc);
     }
-    double re[1] = {acc}, im[1] = {0.0};
-    block_reduce_store<1>(re, im, 1, partial, 1);
-}
-
-// out[j] = sum of partial[j][0..nb)
-__global__ void finalize_kernel(const double2 *__restrict__ partial, size_t pstride, int nb, double2 *__restrict__ out) {
-    const int j = blockIdx.x;
-    double a = 0, b = 0;
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) { double2 t = partial[(size_t)j * pstride + i]; a += t.x; b += t.y; }
-    a = warp_sum(a); b = warp_sum(b);
-    __shared__ double sh[2][32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) { sh[0][w] = a; sh[1][w] = b; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double x = 0, y = 0;
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) { x += sh[0][i]; y += sh[1][i]; }
-        out[j] = make_double2(x, y);
-    }
+    double v[2] = {acc, 0.0};
+    grid_reduce<2>(v, 0, 1, out);
 }
 
 // ---------------------------------------------------------------------------
@@ -210,24 +270,28 @@ __device__ __forceinline__ void ds_mac(float &h, float &l, float uh, float ul, f
 
 constexpr int DS_CHUNK = 8;
 
-__global__ void __launch_bounds__(RED_THREADS) multidot_ds_kernel(PtrPack X, int k, const double2 *__restrict__ y,
-                                                                  size_t n, double2 *__restrict__ partial,
-                                                                  size_t pstride) {
+__global__ void __launch_bounds__(RED_THREADS, 3) multidot_ds_kernel(PtrPack X, int k, int per,
+                                                                     const double2 *__restrict__ y, size_t n, RedOut out) {
+    const int j0 = blockIdx.y * per;
+    k = min(per, k - j0);
     float rh[DS_CHUNK], rl[DS_CHUNK], ih[DS_CHUNK], il[DS_CHUNK];
 #pragma unroll
     for (int j = 0; j < DS_CHUNK; ++j) { rh[j] = rl[j] = ih[j] = il[j] = 0.0f; }
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const double2 b = y[i];
+        double2 a[DS_CHUNK];
+#pragma unroll
+        for (int j = 0; j < DS_CHUNK; ++j)
+            if (j < k) a[j] = static_cast<const double2 *>(X.p[j0 + j])[i];
         float brh, brl, bih, bil;
         ds_split(b.x, brh, brl);
         ds_split(b.y, bih, bil);
 #pragma unroll
         for (int j = 0; j < DS_CHUNK; ++j) {
             if (j < k) {
-                const double2 a = static_cast<const double2 *>(X.p[j])[i];
                 float arh, arl, aih, ail;
-                ds_split(a.x, arh, arl);
-                ds_split(a.y, aih, ail);
+                ds_split(a[j].x, arh, arl);
+                ds_split(a[j].y, aih, ail);
                 // conj(a) b = (ar br + ai bi) + i (ar bi - ai br)
                 ds_mac(rh[j], rl[j], arh, arl, brh, brl);
                 ds_mac(rh[j], rl[j], aih, ail, bih, bil);
@@ -236,126 +300,151 @@ __global__ void __launch_bounds__(RED_THREADS) multidot_ds_kernel(PtrPack X, int
             }
         }
     }
-    double re[DS_CHUNK], im[DS_CHUNK];
+    double v[2 * DS_CHUNK];
 #pragma unroll
     for (int j = 0; j < DS_CHUNK; ++j) {
-        re[j] = f2d_exact(rh[j]) + f2d_exact(rl[j]);
-        im[j] = f2d_exact(ih[j]) + f2d_exact(il[j]);
+        v[2 * j] = f2d_exact(rh[j]) + f2d_exact(rl[j]);
+        v[2 * j + 1] = f2d_exact(ih[j]) + f2d_exact(il[j]);
     }
-    block_reduce_store<DS_CHUNK>(re, im, k, partial, pstride);
+    grid_reduce<2 * DS_CHUNK>(v, j0, k, out);
 }
 
+static RedOut red_out_at(Ctx &c, cpx<double> *d_out) {
+    double2 *p = c.red_partial.as<double2>();
+    return {p, reinterpret_cast<unsigned int *>(p + (size_t)MAXVEC * RED_MAXBLOCKS), reinterpret_cast<double2 *>(d_out)};
+}
+
+template <typename R>
+void blas_multidot(Ctx &c, const void *const *X, int k, const void *y, size_t n, cpx<double> *d_out) {
+    if (k < 1) return;
+    MG_REQUIRE(k <= MAXVEC, MGEIG_EINVAL);
+    const bool ds = sizeof(R) == 8 && c.ds_blas();
+    const int C = ds ? DS_CHUNK : Chunk<R>::n, chunks = (k + C - 1) / C, per = (k + chunks - 1) / chunks;
+    // FP32 vectors below 8 M complex values (a 16^3 x 32 spinor is 1.6 M): 2 blocks
+    // per SM and chunk, 1.3x faster there than 4 (measured); the others 4.  The grid does not
+    // depend on k, so that a thread's sums do not either
+    const int nb = red_grid(c, n, (sizeof(R) == 4 && n < ((size_t)8 << 20)) ? 2 : 4);
+    TimeScope ts(c.timer, sizeof(R) == 8 ? K_BLAS_F64 : K_BLAS_LOW, (double)(k + 1) * n * 2 * sizeof(R));
+    PtrPack pk{};
+    for (int j = 0; j < k; ++j) pk.p[j] = X[j];
+    const RedOut out = red_out_at(c, d_out);
+    if (ds)
+        multidot_ds_kernel<<<dim3(nb, chunks), RED_THREADS, 0, c.stream>>>(pk, k, per, static_cast<const double2 *>(y), n, out);
+    else
+        multidot_kernel<R><<<dim3(nb, chunks), RED_THREADS, 0, c.stream>>>(pk, k, per, y, n, out, vec4_ok<R>(pk, k, y, n));
+    MG_CHECK_LAUNCH();
+}
+
+template <typename R>
+void blas_norm2(Ctx &c, const void *x, size_t n, cpx<double> *d_out) {
+    TimeScope ts(c.timer, sizeof(R) == 8 ? K_BLAS_F64 : K_BLAS_LOW, (double)n * 2 * sizeof(R));
+    norm2_kernel<R><<<red_grid(c, n), RED_THREADS, 0, c.stream>>>(x, n, red_out_at(c, d_out));
+    MG_CHECK_LAUNCH();
+}
+
+void blas_resid_norm2(Ctx &c, const void *qv, const void *v, const cpx<double> *d_lambda, size_t n, cpx<double> *d_out) {
+    TimeScope ts(c.timer, K_BLAS_F64, (double)n * 32);
+    resid_norm2_kernel<<<red_grid(c, n), RED_THREADS, 0, c.stream>>>(
+        static_cast<const double2 *>(qv), static_cast<const double2 *>(v), reinterpret_cast<const double2 *>(d_lambda), n,
+        red_out_at(c, d_out));
+    MG_CHECK_LAUNCH();
+}
+
+// The coefficients of an update: in device memory (results of a reduction) or, for
+// callers that hold them on the host, in the launch's parameters
+struct DevCoef {
+    const double2 *p;
+    __device__ __forceinline__ double2 operator[](int j) const { return p[j]; }
+};
+constexpr int HOST_COEFS = 32;
+struct HostCoef {
+    double2 v[HOST_COEFS];
+    __device__ __forceinline__ double2 operator[](int j) const { return v[j]; }
+};
+
+// vectors of an update that are loaded before they are used
+constexpr int AXPY_BATCH = 8;
+
 // y += sign * sum_j coef[j] X_j, y and X_j FP64, double-float arithmetic
-__global__ void __launch_bounds__(256) multi_axpy_ds_kernel(double2 *__restrict__ y, PtrPack X, int k,
-                                                            const double2 *__restrict__ coef, double sign, size_t n) {
-    float crh[DS_CHUNK], crl[DS_CHUNK], cih[DS_CHUNK], cil[DS_CHUNK];
-#pragma unroll
-    for (int j = 0; j < DS_CHUNK; ++j) {
-        if (j < k) {
-            const double2 t = coef[j];
-            ds_split(sign * t.x, crh[j], crl[j]);
-            ds_split(sign * t.y, cih[j], cil[j]);
-        } else {
-            crh[j] = crl[j] = cih[j] = cil[j] = 0.0f;
-        }
+template <typename Coef>
+__global__ void __launch_bounds__(256) multi_axpy_ds_kernel(double2 *__restrict__ y, PtrPack X, int k, Coef coef,
+                                                            double sign, size_t n) {
+    __shared__ float4 cf[MAXVEC];   // (re high, re low, im high, im low)
+    if (threadIdx.x < k) {
+        const double2 t = coef[threadIdx.x];
+        float4 f;
+        ds_split(sign * t.x, f.x, f.y);
+        ds_split(sign * t.y, f.z, f.w);
+        cf[threadIdx.x] = f;
     }
+    __syncthreads();
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const double2 t = y[i];
         float rh, rl, ih, il;
         ds_split(t.x, rh, rl);
         ds_split(t.y, ih, il);
+        for (int j0 = 0; j0 < k; j0 += AXPY_BATCH) {
+            double2 a[AXPY_BATCH];
 #pragma unroll
-        for (int j = 0; j < DS_CHUNK; ++j) {
-            if (j < k) {
-                const double2 a = static_cast<const double2 *>(X.p[j])[i];
-                float arh, arl, aih, ail;
-                ds_split(a.x, arh, arl);
-                ds_split(a.y, aih, ail);
-                // c a = (cr ar - ci ai) + i (cr ai + ci ar)
-                ds_mac(rh, rl, crh[j], crl[j], arh, arl);
-                ds_mac(rh, rl, -cih[j], -cil[j], aih, ail);
-                ds_mac(ih, il, crh[j], crl[j], aih, ail);
-                ds_mac(ih, il, cih[j], cil[j], arh, arl);
+            for (int j = 0; j < AXPY_BATCH; ++j)
+                if (j0 + j < k) a[j] = static_cast<const double2 *>(X.p[j0 + j])[i];
+            if (j0) {   // y is rounded to FP64 after every eight vectors
+                ds_split(f2d_exact(rh) + f2d_exact(rl), rh, rl);
+                ds_split(f2d_exact(ih) + f2d_exact(il), ih, il);
+            }
+#pragma unroll
+            for (int j = 0; j < AXPY_BATCH; ++j) {
+                if (j0 + j < k) {
+                    float arh, arl, aih, ail;
+                    ds_split(a[j].x, arh, arl);
+                    ds_split(a[j].y, aih, ail);
+                    const float4 c = cf[j0 + j];
+                    // c a = (cr ar - ci ai) + i (cr ai + ci ar)
+                    ds_mac(rh, rl, c.x, c.y, arh, arl);
+                    ds_mac(rh, rl, -c.z, -c.w, aih, ail);
+                    ds_mac(ih, il, c.x, c.y, aih, ail);
+                    ds_mac(ih, il, c.z, c.w, arh, arl);
+                }
             }
         }
         y[i] = make_double2(f2d_exact(rh) + f2d_exact(rl), f2d_exact(ih) + f2d_exact(il));
     }
 }
 
-static double2 *partial_ptr(Ctx &c) { return c.red_partial.as<double2>(); }
-
-template <typename R>
-void blas_multidot(Ctx &c, const void *const *X, int k, const void *y, size_t n, cpx<double> *d_out) {
-    // FP32 vectors below 8 M complex values (a 16^3 x 32 spinor is 1.6 M): 2 blocks
-    // per SM, 1.3x faster there than 4 (measured); the longer ones and the
-    // double-float kernels run best at 4
-    const int nb = red_grid(c, n, (sizeof(R) == 4 && n < ((size_t)8 << 20)) ? 2 : 4);
-    const size_t pstride = RED_MAXBLOCKS;
-    TimeScope ts(c.timer, sizeof(R) == 8 ? K_BLAS_F64 : K_BLAS_LOW, (double)(k + 1) * n * 2 * sizeof(R));
-    const bool ds = sizeof(R) == 8 && c.ds_blas();
-    const int C = ds ? DS_CHUNK : Chunk<R>::n;
-    for (int j0 = 0; j0 < k; j0 += C) {
-        PtrPack pk{};
-        const int kk = k - j0 < C ? k - j0 : C;
-        for (int j = 0; j < kk; ++j) pk.p[j] = X[j0 + j];
-        if (ds)
-            multidot_ds_kernel<<<nb, RED_THREADS, 0, c.stream>>>(pk, kk, static_cast<const double2 *>(y), n,
-                                                                  partial_ptr(c) + (size_t)j0 * pstride, pstride);
-        else
-            multidot_kernel<R><<<nb, RED_THREADS, 0, c.stream>>>(pk, kk, y, n, partial_ptr(c) + (size_t)j0 * pstride,
-                                                                 pstride, vec4_ok<R>(pk, kk, y, n));
-        MG_CHECK_LAUNCH();
-    }
-    finalize_kernel<<<k, 128, 0, c.stream>>>(partial_ptr(c), pstride, nb, reinterpret_cast<double2 *>(d_out));
-    MG_CHECK_LAUNCH();
-}
-
-template <typename R>
-void blas_norm2(Ctx &c, const void *x, size_t n, cpx<double> *d_out) {
-    const int nb = red_grid(c, n);
-    TimeScope ts(c.timer, sizeof(R) == 8 ? K_BLAS_F64 : K_BLAS_LOW, (double)n * 2 * sizeof(R));
-    norm2_kernel<R><<<nb, RED_THREADS, 0, c.stream>>>(x, n, partial_ptr(c));
-    MG_CHECK_LAUNCH();
-    finalize_kernel<<<1, 128, 0, c.stream>>>(partial_ptr(c), RED_MAXBLOCKS, nb, reinterpret_cast<double2 *>(d_out));
-    MG_CHECK_LAUNCH();
-}
-
-void blas_resid_norm2(Ctx &c, const void *qv, const void *v, const cpx<double> *d_lambda, size_t n, cpx<double> *d_out) {
-    const int nb = red_grid(c, n);
-    TimeScope ts(c.timer, K_BLAS_F64, (double)n * 32);
-    resid_norm2_kernel<<<nb, RED_THREADS, 0, c.stream>>>(static_cast<const double2 *>(qv), static_cast<const double2 *>(v),
-                                                         reinterpret_cast<const double2 *>(d_lambda), n, partial_ptr(c));
-    MG_CHECK_LAUNCH();
-    finalize_kernel<<<1, 128, 0, c.stream>>>(partial_ptr(c), RED_MAXBLOCKS, nb, reinterpret_cast<double2 *>(d_out));
-    MG_CHECK_LAUNCH();
-}
-
 // y += sign * sum_j coef[j] X_j
-template <typename R>
-__global__ void multi_axpy_kernel(void *__restrict__ yv, PtrPack X, int k, const double2 *__restrict__ coef, double sign,
-                                  size_t n, bool vec4) {
+template <typename R, typename Coef>
+__global__ void __launch_bounds__(256) multi_axpy_kernel(void *__restrict__ yv, PtrPack X, int k, Coef coef, double sign,
+                                                         size_t n, bool vec4) {
     typedef typename V2<R>::T T;
     T *y = static_cast<T *>(yv);
-    constexpr int C = Chunk<R>::n;
-    R cr[C], ci[C];
-#pragma unroll
-    for (int j = 0; j < C; ++j) {
-        if (j < k) { double2 t = coef[j]; cr[j] = (R)(sign * t.x); ci[j] = (R)(sign * t.y); }
-        else { cr[j] = 0; ci[j] = 0; }
+    __shared__ T cf[MAXVEC];
+    if (threadIdx.x < k) {
+        const double2 t = coef[threadIdx.x];
+        T f;
+        f.x = (R)(sign * t.x);
+        f.y = (R)(sign * t.y);
+        cf[threadIdx.x] = f;
     }
+    __syncthreads();
     if constexpr (sizeof(R) == 4) {
         if (vec4) {   // two complex values per 16-byte access
             float4 *y4 = static_cast<float4 *>(yv);
             for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n / 2; i += (size_t)gridDim.x * blockDim.x) {
                 float4 acc = y4[i];
+                for (int j0 = 0; j0 < k; j0 += AXPY_BATCH) {
+                    float4 a[AXPY_BATCH];
 #pragma unroll
-                for (int j = 0; j < C; ++j) {
-                    if (j < k) {
-                        const float4 a = static_cast<const float4 *>(X.p[j])[i];
-                        acc.x = fmaf(cr[j], a.x, acc.x); acc.x = fmaf(-ci[j], a.y, acc.x);
-                        acc.y = fmaf(cr[j], a.y, acc.y); acc.y = fmaf(ci[j], a.x, acc.y);
-                        acc.z = fmaf(cr[j], a.z, acc.z); acc.z = fmaf(-ci[j], a.w, acc.z);
-                        acc.w = fmaf(cr[j], a.w, acc.w); acc.w = fmaf(ci[j], a.z, acc.w);
+                    for (int j = 0; j < AXPY_BATCH; ++j)
+                        if (j0 + j < k) a[j] = static_cast<const float4 *>(X.p[j0 + j])[i];
+#pragma unroll
+                    for (int j = 0; j < AXPY_BATCH; ++j) {
+                        if (j0 + j < k) {
+                            const T c = cf[j0 + j];
+                            acc.x = fmaf(c.x, a[j].x, acc.x); acc.x = fmaf(-c.y, a[j].y, acc.x);
+                            acc.y = fmaf(c.x, a[j].y, acc.y); acc.y = fmaf(c.y, a[j].x, acc.y);
+                            acc.z = fmaf(c.x, a[j].z, acc.z); acc.z = fmaf(-c.y, a[j].w, acc.z);
+                            acc.w = fmaf(c.x, a[j].w, acc.w); acc.w = fmaf(c.y, a[j].z, acc.w);
+                        }
                     }
                 }
                 y4[i] = acc;
@@ -365,12 +454,18 @@ __global__ void multi_axpy_kernel(void *__restrict__ yv, PtrPack X, int k, const
     }
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         T acc = y[i];
+        for (int j0 = 0; j0 < k; j0 += AXPY_BATCH) {
+            T a[AXPY_BATCH];
 #pragma unroll
-        for (int j = 0; j < C; ++j) {
-            if (j < k) {
-                T a = static_cast<const T *>(X.p[j])[i];
-                acc.x = fma(cr[j], a.x, acc.x); acc.x = fma(-ci[j], a.y, acc.x);
-                acc.y = fma(cr[j], a.y, acc.y); acc.y = fma(ci[j], a.x, acc.y);
+            for (int j = 0; j < AXPY_BATCH; ++j)
+                if (j0 + j < k) a[j] = static_cast<const T *>(X.p[j0 + j])[i];
+#pragma unroll
+            for (int j = 0; j < AXPY_BATCH; ++j) {
+                if (j0 + j < k) {
+                    const T c = cf[j0 + j];
+                    acc.x = fma(c.x, a[j].x, acc.x); acc.x = fma(-c.y, a[j].y, acc.x);
+                    acc.y = fma(c.x, a[j].y, acc.y); acc.y = fma(c.y, a[j].x, acc.y);
+                }
             }
         }
         y[i] = acc;
@@ -387,26 +482,38 @@ static int ew_grid(const Ctx &c, size_t n, int per_sm = 16) {
     return (int)(b < cap ? (b < 1 ? 1 : b) : cap);
 }
 
+template <typename R, typename Coef>
+static void launch_multi_axpy(Ctx &c, void *y, const void *const *X, int k, const Coef &coef, double sign, size_t n) {
+    MG_REQUIRE(k <= MAXVEC, MGEIG_EINVAL);
+    TimeScope ts(c.timer, sizeof(R) == 8 ? K_BLAS_F64 : K_BLAS_LOW, (double)(k + 2) * n * 2 * sizeof(R));
+    PtrPack pk{};
+    for (int j = 0; j < k; ++j) pk.p[j] = X[j];
+    if (sizeof(R) == 8 && c.ds_blas()) {
+        multi_axpy_ds_kernel<<<ew_grid(c, n), 256, 0, c.stream>>>(static_cast<double2 *>(y), pk, k, coef, sign, n);
+    } else {
+        const bool v4 = vec4_ok<R>(pk, k, y, n);
+        multi_axpy_kernel<R><<<ew_grid(c, v4 ? n / 2 : n, sizeof(R) == 4 ? 4 : 16), 256, 0, c.stream>>>(y, pk, k, coef,
+                                                                                                        sign, n, v4);
+    }
+    MG_CHECK_LAUNCH();
+}
+
 template <typename R>
 void blas_multi_axpy(Ctx &c, void *y, const void *const *X, int k, const cpx<double> *d_coef, double sign, size_t n) {
-    TimeScope ts(c.timer, sizeof(R) == 8 ? K_BLAS_F64 : K_BLAS_LOW, (double)(k + 2) * n * 2 * sizeof(R));
-    const bool ds = sizeof(R) == 8 && c.ds_blas();
-    const int C = ds ? DS_CHUNK : Chunk<R>::n;
-    for (int j0 = 0; j0 < k; j0 += C) {
-        PtrPack pk{};
-        const int kk = k - j0 < C ? k - j0 : C;
-        for (int j = 0; j < kk; ++j) pk.p[j] = X[j0 + j];
-        if (ds) {
-            multi_axpy_ds_kernel<<<ew_grid(c, n), 256, 0, c.stream>>>(
-                static_cast<double2 *>(y), pk, kk, reinterpret_cast<const double2 *>(d_coef + j0), sign, n);
-        } else {
-            const bool v4 = vec4_ok<R>(pk, kk, y, n);
-            multi_axpy_kernel<R><<<ew_grid(c, v4 ? n / 2 : n, sizeof(R) == 4 ? 4 : 16), 256, 0, c.stream>>>(
-                y, pk, kk, reinterpret_cast<const double2 *>(d_coef + j0), sign, n, v4);
-        }
-        MG_CHECK_LAUNCH();
-    }
+    if (k < 1) return;
+    launch_multi_axpy<R>(c, y, X, k, DevCoef{reinterpret_cast<const double2 *>(d_coef)}, sign, n);
 }
+
+// k <= 32 coefficients from the host, in the launch's parameters (no upload)
+template <typename R>
+void blas_multi_axpy_host(Ctx &c, void *y, const void *const *X, int k, const double *coef, size_t n) {
+    MG_REQUIRE(k >= 1 && k <= HOST_COEFS, MGEIG_EINVAL);
+    HostCoef h;
+    for (int j = 0; j < k; ++j) h.v[j] = make_double2(coef[2 * j], coef[2 * j + 1]);
+    launch_multi_axpy<R>(c, y, X, k, h, 1.0, n);
+}
+template void blas_multi_axpy_host<double>(Ctx &, void *, const void *const *, int, const double *, size_t);
+template void blas_multi_axpy_host<float>(Ctx &, void *, const void *const *, int, const double *, size_t);
 
 template <typename R>
 __global__ void axpy_kernel(double ar, double ai, const void *__restrict__ xv, void *__restrict__ yv, size_t n) {

@@ -90,17 +90,21 @@ __host__ __device__ __forceinline__ dsf fma(dsf a, dsf b, dsf c) { return a * b 
 // the low word is dropped below 2^-80, |d| >= 2^128 gives +-inf.
 __device__ __forceinline__ void ds_split(double d, float &hi, float &lo) {
     const unsigned hw = (unsigned)__double2hiint(d), lw = (unsigned)__double2loint(d);
-    const unsigned sgn = hw & 0x80000000u;
-    const unsigned e = (hw >> 20) & 0x7ffu;   // biased FP64 exponent
+    const unsigned sgn = hw & 0x80000000u, t = hw ^ sgn;   // t: the magnitude's high word, exponent in bits 20..30
     // FP32 exponent field e - 896; the top 23 mantissa bits: 20 of hw, 3 of lw
-    unsigned hb = __funnelshift_l(lw, (hw & 0x7fffffffu) - (896u << 20), 3) | sgn;
-    hb = e < 897u ? sgn : hb;
-    hb = e > 1150u ? (sgn | 0x7f800000u) : hb;
-    hi = __uint_as_float(hb);
+    unsigned hb = __funnelshift_l(lw, t - (896u << 20), 3) | sgn;
     // lo = m * 2^(e - 1023 - 46) for the next 23 mantissa bits m = lw[28:6]:
     // x = 2^23 + m exactly (the mantissa field of 2^23), lo = x s - 2^23 s
     const float x = __uint_as_float(0x4B000000u | ((lw >> 6) & 0x7fffffu));
-    const float sc = (e >= 943u && e <= 1150u) ? __uint_as_float(sgn | ((e - 942u) << 23)) : 0.0f;
+    unsigned sb = (((t - (942u << 20)) << 3) & 0x7f800000u) | sgn;
+    if (t - (943u << 20) >= (208u << 20)) {   // outside 2^-80 .. 2^128: rare, so one test on the usual path
+        const unsigned e = t >> 20;           // biased FP64 exponent
+        hb = e < 897u ? sgn : hb;
+        hb = e > 1150u ? (sgn | 0x7f800000u) : hb;
+        sb = 0u;
+    }
+    const float sc = __uint_as_float(sb);
+    hi = __uint_as_float(hb);
     lo = fmaf(x, sc, -__fmul_rn(sc, 8388608.0f));
 }
 

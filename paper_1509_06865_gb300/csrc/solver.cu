@@ -103,7 +103,10 @@ constexpr int H1 = 0, H2 = 128, HN = 256, CGS = 257, NFETCH = 258, UP = 300;
 void ensure_reduction(Ctx &c, int max_vectors) {
     (void)max_vectors;
     if (!c.red_partial.p) {
-        c.red_partial.alloc((size_t)(MAX_ITERATED + 8) * 1024 * sizeof(double2));   // >= (vectors + 1) x 1024 blocks
+        // (vectors + 1) x 1024 blocks of partial sums, then the reductions' tickets (zero between launches)
+        const size_t part = (size_t)(MAX_ITERATED + 8) * 1024 * sizeof(double2);
+        c.red_partial.alloc(part + 256);
+        MG_CUDA(cudaMemset(c.red_partial.as<char>() + part, 0, 256));
         c.red_out.alloc(RED_SLOTS * sizeof(double2));
         MG_CUDA(cudaMemset(c.red_out.p, 0, RED_SLOTS * sizeof(double2)));
         MG_CUDA(cudaMallocHost(&c.pinned, 2 * RED_SLOTS * sizeof(double2)));
@@ -159,10 +162,8 @@ void blas_dot_host(Ctx &c, bool f32, int k, const void *const *X, const void *y,
 
 void blas_axpy_host(Ctx &c, bool f32, int k, const void *const *X, const double *coef, void *y, size_t n) {
     ensure_reduction(c, k);
-    std::vector<cpx<double>> cv(k);
-    for (int j = 0; j < k; ++j) cv[j] = cpx<double>(coef[2 * j], coef[2 * j + 1]);
-    if (f32) blas_multi_axpy<float>(c, y, X, k, upload(c, cv), 1.0, n);
-    else blas_multi_axpy<double>(c, y, X, k, upload(c, cv), 1.0, n);
+    if (f32) blas_multi_axpy_host<float>(c, y, X, k, coef, n);
+    else blas_multi_axpy_host<double>(c, y, X, k, coef, n);
     sync(c);
 }
 

@@ -561,8 +561,7 @@ int mgeig_coarse_apply_nrhs(mgeig_ctx *ctx, double sigma, const double *xc, doub
             coarse_apply_nrhs(c, sigma, a32.p, b32.p, nrhs);
             coarse_flat_convert(c, b32.p, b.p, n * nrhs, false);
         } else {
-            for (int r = 0; r < nrhs; ++r)
-                coarse_apply<double>(c, c.Dc.p, sigma, a.as<char>() + n * 16 * r, b.as<char>() + n * 16 * r, false);
+            coarse_apply_many<double>(c, sigma, a.p, b.p, nrhs);
         }
         MG_CUDA(cudaMemcpyAsync(yc, b.p, b64, cudaMemcpyDeviceToHost, c.stream));
         sync(c);

@@ -143,13 +143,14 @@ template <typename R> void build_interp(Ctx &c, const void *const *W64, int ntv,
 template <typename R> void restrict_vec(Ctx &c, const void *const *P, const void *r, void *rc);
 template <typename R> void prolong_vec(Ctx &c, const void *const *P, const void *ec, void *e);
 template <typename R> void build_coarse(Ctx &c, const void *const *P, void *Dc);
-template <typename R> void coarse_apply(Ctx &c, const void *Dc, double sigma, const void *x, void *y, bool dform = false);
-template <typename R> void coarse_gamma5(Ctx &c, const void *x, void *y);
+template <typename R> void coarse_apply(Ctx &c, double sigma, const void *x, void *y);
+// n vectors back to back, the operator in the level precision
+template <typename R> void coarse_apply_many(Ctx &c, double sigma, const void *X, void *Y, int n);
 template <typename R> void sap_sweep(Ctx &c, int colour, double sigma, const void *rhs, bool rhs_gamma5, void *z);
 
 // ----- 16-bit coarse links (links16.cu) -----
 void compress_coarse(Ctx &c);   // Dc (FP32) -> Dc16, Dcs in the format of prm.coarse_links
-void coarse_apply_links16(Ctx &c, double sigma, const void *x, void *y, bool dform);
+void coarse_apply_links16(Ctx &c, double sigma, const void *x, void *y);
 // Y = (Q_c - sigma) X for nrhs <= 16 FP32 coarse vectors back to back (tensor cores with BF16 links)
 void coarse_apply_nrhs(Ctx &c, double sigma, const void *X, void *Y, int nrhs);
 // n flat complex values FP64 -> FP32 (to32) or back (solver.cu)

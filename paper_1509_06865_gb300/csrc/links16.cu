@@ -6,8 +6,8 @@
 //   compress_coarse        FP32 blocks Dc[d][site][col][row] -> 16-bit planes
 //                          L[d][site][re|im][row][col] (entries divided by the
 //                          block's largest |re|, |im|) and scale[d][site]
-//   coarse_apply_links16   y = (Q_c - sigma) x (or the D_c form), one right-hand
-//                          side, thread per coarse row
+//   coarse_apply_links16   y = (Q_c - sigma) x, one right-hand side, thread per
+//                          coarse row
 //   coarse_apply_nrhs      Y = (Q_c - sigma) X for nrhs <= 16 right-hand sides
 //                          on the tensor cores (mma.sync m16n8k16, BF16 in, FP32
 //                          accumulate): per coarse site
@@ -73,7 +73,7 @@ void compress_coarse(Ctx &c) {
 template <typename H>
 __global__ void coarse_apply16_kernel(int nagg, int ntv, const H *__restrict__ L, const float *__restrict__ scale,
                                       const int *__restrict__ nbr, float sigma, const float2 *__restrict__ x,
-                                      float2 *__restrict__ y, int dform) {
+                                      float2 *__restrict__ y) {
     using HP = typename H16<H>::P;
     const int n2 = 2 * ntv;
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -100,16 +100,11 @@ __global__ void coarse_apply16_kernel(int nagg, int ntv, const H *__restrict__ L
         ai = fmaf(s, di, ai);
     }
     const float2 xt = x[t];
-    if (dform) {
-        const float sg = row >= ntv ? -sigma : sigma;
-        y[t] = make_float2(ar - sg * xt.x, ai - sg * xt.y);
-    } else {
-        if (row >= ntv) { ar = -ar; ai = -ai; }
-        y[t] = make_float2(ar - sigma * xt.x, ai - sigma * xt.y);
-    }
+    if (row >= ntv) { ar = -ar; ai = -ai; }
+    y[t] = make_float2(ar - sigma * xt.x, ai - sigma * xt.y);
 }
 
-void coarse_apply_links16(Ctx &c, double sigma, const void *x, void *y, bool dform) {
+void coarse_apply_links16(Ctx &c, double sigma, const void *x, void *y) {
     const int ntv = c.prm.n_tv, n2 = 2 * ntv;
     MG_REQUIRE(n2 % 2 == 0 && c.Dc16.p && c.cnbr.p, MGEIG_ENOTSETUP);
     const size_t n = (size_t)c.nagg * n2;
@@ -117,11 +112,11 @@ void coarse_apply_links16(Ctx &c, double sigma, const void *x, void *y, bool dfo
     if (c.prm.coarse_links == MGEIG_LINKS_BF16)
         coarse_apply16_kernel<__nv_bfloat16><<<grid_for(n, 128), 128, 0, c.stream>>>(
             c.nagg, ntv, c.Dc16.as<__nv_bfloat16>(), c.Dcs.as<float>(), c.cnbr.as<int>(), (float)sigma,
-            static_cast<const float2 *>(x), static_cast<float2 *>(y), dform ? 1 : 0);
+            static_cast<const float2 *>(x), static_cast<float2 *>(y));
     else
         coarse_apply16_kernel<__half><<<grid_for(n, 128), 128, 0, c.stream>>>(
             c.nagg, ntv, c.Dc16.as<__half>(), c.Dcs.as<float>(), c.cnbr.as<int>(), (float)sigma,
-            static_cast<const float2 *>(x), static_cast<float2 *>(y), dform ? 1 : 0);
+            static_cast<const float2 *>(x), static_cast<float2 *>(y));
     MG_CHECK_LAUNCH();
 }
 
@@ -292,14 +287,14 @@ void coarse_apply_nrhs(Ctx &c, double sigma, const void *X, void *Y, int nrhs) {
     MG_REQUIRE(nrhs >= 1 && nrhs <= TC_MAXN, MGEIG_EINVAL);
     MG_REQUIRE(c.cnbr.p && c.Dc.p, MGEIG_ENOTSETUP);
     const size_t vb = (size_t)c.nagg * n2 * sizeof(float2);
-    if (c.prm.coarse_links != MGEIG_LINKS_BF16) {
-        // FP32 or FP16 links: the CUDA-core kernels, one right-hand side after another
-        for (int r = 0; r < nrhs; ++r) {
-            const void *xr = static_cast<const char *>(X) + vb * r;
-            void *yr = static_cast<char *>(Y) + vb * r;
-            if (c.prm.coarse_links == MGEIG_LINKS_F16) coarse_apply_links16(c, sigma, xr, yr, false);
-            else coarse_apply<float>(c, c.Dc.p, sigma, xr, yr, false);
-        }
+    if (c.prm.coarse_links == MGEIG_LINKS_LEVEL) {
+        coarse_apply_many<float>(c, sigma, X, Y, nrhs);
+        return;
+    }
+    if (c.prm.coarse_links == MGEIG_LINKS_F16) {
+        // the CUDA-core kernel, one right-hand side after another
+        for (int r = 0; r < nrhs; ++r)
+            coarse_apply_links16(c, sigma, static_cast<const char *>(X) + vb * r, static_cast<char *>(Y) + vb * r);
         return;
     }
     MG_REQUIRE(n2 <= 48 && c.Dc16.p, MGEIG_EINVAL);

@@ -482,9 +482,11 @@ static void deflation_prepare(Ctx &c, double sigma) {
     const size_t n = c.coarse_ncpx(), vb = cR_bytes(c);
     std::vector<const void *> Wp(k);
     for (int i = 0; i < k; ++i) Wp[i] = static_cast<const char *>(w.Wc.p) + vb * i;
+    const bool level = sizeof(R) == 8 || c.prm.coarse_links == MGEIG_LINKS_LEVEL;
+    if (level) coarse_apply_many<R>(c, sigma, w.Wc.p, w.AWc.p, k);
     for (int j = 0; j < k; ++j) {
         void *awj = static_cast<char *>(w.AWc.p) + vb * j;
-        coarse_apply<R>(c, c.Dc.p, sigma, Wp[j], awj, false);
+        if (!level) coarse_apply<R>(c, sigma, Wp[j], awj);
         blas_multidot<R>(c, Wp.data(), k, awj, n, w.Edev.as<cpx<double>>() + (size_t)j * k);
     }
     std::vector<cpx<double>> Ecol((size_t)k * k), E((size_t)k * k), Ei;
@@ -1478,8 +1480,8 @@ static void coarse_out(Ctx &c, const void *xR, void *x64) {
 void coarse_apply_f64(Ctx &c, double sigma, const void *x64, void *y64) {
     Ctx::Work &w = *c.work;
     coarse_in(c, x64, w.rc.p);
-    if (c.mixed()) coarse_apply<float>(c, c.Dc.p, sigma, w.rc.p, w.ec.p);
-    else coarse_apply<double>(c, c.Dc.p, sigma, w.rc.p, w.ec.p);
+    if (c.mixed()) coarse_apply<float>(c, sigma, w.rc.p, w.ec.p);
+    else coarse_apply<double>(c, sigma, w.rc.p, w.ec.p);
     coarse_out(c, w.ec.p, y64);
 }
 
@@ -1634,9 +1636,11 @@ static void deflation_prepare_fixed(Ctx &c, double sigma) {
     const size_t n = c.coarse_ncpx(), vb = cR_bytes(c);
     const void *Wp[KMAX];
     for (int i = 0; i < k; ++i) Wp[i] = static_cast<const char *>(w.Wc.p) + vb * i;
+    const bool level = sizeof(R) == 8 || c.prm.coarse_links == MGEIG_LINKS_LEVEL;
+    if (level) coarse_apply_many<R>(c, sigma, w.Wc.p, w.AWc.p, k);
     for (int j = 0; j < k; ++j) {
         void *awj = static_cast<char *>(w.AWc.p) + vb * j;
-        coarse_apply<R>(c, c.Dc.p, sigma, Wp[j], awj, false);
+        if (!level) coarse_apply<R>(c, sigma, Wp[j], awj);
         blas_multidot<R>(c, Wp, k, awj, n, w.Edev.as<cpx<double>>() + (size_t)j * k);
     }
     cpx<double> Ecol[KMAX * KMAX], E[KMAX * KMAX], Ei[KMAX * KMAX];

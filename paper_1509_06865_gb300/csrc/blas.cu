@@ -24,7 +24,8 @@ namespace mgeig {
 
 constexpr int RED_THREADS = 256;
 constexpr int RED_MAXBLOCKS = 1024;
-constexpr int MAXVEC = MAX_ITERATED + 8;   // pointer slots per launch
+constexpr int MAXVEC = MAX_ITERATED + 8;   // pointer slots per launch; more vectors take more launches
+static_assert(MAXVEC % 8 == 0, "a double-float update is rounded after every eight vectors");
 // vectors that share one read of y: 16 in FP32 (bandwidth bound); 8 in FP64, where the
 // FP64 pipe bounds the kernel and 16 accumulators cost occupancy
 template <typename R> struct Chunk { static constexpr int n = sizeof(R) == 4 ? 16 : 8; };
@@ -316,8 +317,8 @@ static RedOut red_out_at(Ctx &c, cpx<double> *d_out) {
 
 template <typename R>
 void blas_multidot(Ctx &c, const void *const *X, int k, const void *y, size_t n, cpx<double> *d_out) {
+    for (; k > MAXVEC; k -= MAXVEC, X += MAXVEC, d_out += MAXVEC) blas_multidot<R>(c, X, MAXVEC, y, n, d_out);
     if (k < 1) return;
-    MG_REQUIRE(k <= MAXVEC, MGEIG_EINVAL);
     const bool ds = sizeof(R) == 8 && c.ds_blas();
     const int C = ds ? DS_CHUNK : Chunk<R>::n, chunks = (k + C - 1) / C, per = (k + chunks - 1) / chunks;
     // FP32 vectors below 8 M complex values (a 16^3 x 32 spinor is 1.6 M): 2 blocks
@@ -484,7 +485,6 @@ static int ew_grid(const Ctx &c, size_t n, int per_sm = 16) {
 
 template <typename R, typename Coef>
 static void launch_multi_axpy(Ctx &c, void *y, const void *const *X, int k, const Coef &coef, double sign, size_t n) {
-    MG_REQUIRE(k <= MAXVEC, MGEIG_EINVAL);
     TimeScope ts(c.timer, sizeof(R) == 8 ? K_BLAS_F64 : K_BLAS_LOW, (double)(k + 2) * n * 2 * sizeof(R));
     PtrPack pk{};
     for (int j = 0; j < k; ++j) pk.p[j] = X[j];
@@ -500,8 +500,8 @@ static void launch_multi_axpy(Ctx &c, void *y, const void *const *X, int k, cons
 
 template <typename R>
 void blas_multi_axpy(Ctx &c, void *y, const void *const *X, int k, const cpx<double> *d_coef, double sign, size_t n) {
-    if (k < 1) return;
-    launch_multi_axpy<R>(c, y, X, k, DevCoef{reinterpret_cast<const double2 *>(d_coef)}, sign, n);
+    for (; k > 0; k -= MAXVEC, X += MAXVEC, d_coef += MAXVEC)
+        launch_multi_axpy<R>(c, y, X, std::min(k, MAXVEC), DevCoef{reinterpret_cast<const double2 *>(d_coef)}, sign, n);
 }
 
 // k <= 32 coefficients from the host, in the launch's parameters (no upload)

@@ -149,3 +149,22 @@ def test_inner_products_and_updates(k, n, prec):
     ctx.multi_axpy_dev(p, c, yd.data_ptr(), n, P)
     assert np.all(np.abs(yd.cpu().numpy() - (y64 + c @ X64)) <= bound * (np.abs(y64) + np.abs(c) @ np.abs(X64)))
     ctx.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["fp64", "mixed"])
+def test_solve_with_a_basis_of_more_vectors_than_a_launch_takes(prec):
+    """FGMRES minimises the residual over its whole basis, so 100 steps without a restart end
+    no further from the solution than 70.  sigma lies deep inside the spectrum, where the
+    cycle is a poor preconditioner, and 1e-13 is out of reach."""
+    name = "ntv3"
+    U, op, W, P, C = oracle_parts(name)
+    b = synth.gaussian_vectors(SHAPES[name]["dims"], 1, 23)[0]
+    res = {}
+    for steps in (70, 100):
+        ctx = make(name, prec, outer_restart=100, outer_maxiter=steps)
+        ctx.set_test_vectors(W)
+        x, st = ctx.solve(b, 1.7, 1e-13)
+        assert st["outer_iters"] == steps and not st["converged"]
+        res[steps] = np.linalg.norm(b - op.Q_sigma(x, 1.7)) / np.linalg.norm(b)
+        ctx.close()
+    assert res[100] <= res[70] * (1 + 1e-6)

@@ -583,20 +583,16 @@ void coarse_apply(Ctx &c, double sigma, const void *x, void *y) {
 // FP32: the block's forward links (two rows, 3 float4 per link) are staged in
 // shared memory once and serve every MR step (the backward link of an in-block
 // hop is the forward link of the in-block neighbour); two CTAs fit an SM.
-template <typename R> struct SapBounds { static constexpr int minb = 1; };
-template <> struct SapBounds<float> { static constexpr int minb = 2; };
-
-template <typename R>
-__global__ void __launch_bounds__(256, SapBounds<R>::minb)
-sap_kernel(Geom g, AggGeom B, int colour, R sigma, const void *__restrict__ U,
+__global__ void __launch_bounds__(256, 2)
+sap_f32_kernel(Geom g, AggGeom B, int colour, float sigma, const void *__restrict__ U,
            const void *__restrict__ clov, const void *__restrict__ rhs, int rhs_g5, void *z, int mr_iters) {
-    extern __shared__ unsigned char smem_raw[];
+    using R = float;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     // component-major (rho[k][vol], slink[mu][3][vol]): consecutive threads read
     // consecutive words, without the 4-way bank conflicts of a site-major layout
     cpx<R> *rho = reinterpret_cast<cpx<R> *>(smem_raw);       // [12][vol]
     float4 *slink = reinterpret_cast<float4 *>(smem_raw + (size_t)B.vol * 12 * sizeof(cpx<R>));   // [4][3][vol]
     const int bv = B.vol;
-    constexpr bool stage = sizeof(R) == 4;
     __shared__ R red[3 * 32];   // MR step sums, in the kernel's precision
     // the grid covers the blocks of one colour: blocks 2i and 2i + 1 differ in
     // colour (an even number of blocks per direction), CTA i takes the one of
@@ -618,7 +614,7 @@ sap_kernel(Geom g, AggGeom B, int colour, R sigma, const void *__restrict__ U,
     cpx<R> e[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) e[k] = cpx<R>();
-    if (stage && active) {
+    if (active) {
         const float4 *ug = static_cast<const float4 *>(U);
         for (int mu = 0; mu < 4; ++mu)
             for (int e = 0; e < 3; ++e) slink[(mu * 3 + e) * bv + l] = ug[((size_t)mu * 3 + e) * V + s];
@@ -675,19 +671,13 @@ sap_kernel(Geom g, AggGeom B, int colour, R sigma, const void *__restrict__ U,
                     int ln = l + (fwd ? 1 : -1) * (mu == 0 ? 1 : mu == 1 ? B.agg[0] : mu == 2 ? B.agg[0] * B.agg[1]
                                                                                               : B.agg[0] * B.agg[1] * B.agg[2]);
                     cpx<R> u[9], psi[12];
-                    if constexpr (stage) {
-                        const float4 *q = slink + (size_t)mu * 3 * bv + (fwd ? l : ln);
-                        const float4 a = q[0], b = q[bv], cc = q[2 * bv];
-                        u[0] = cpx<R>(a.x, a.y); u[1] = cpx<R>(a.z, a.w); u[2] = cpx<R>(b.x, b.y);
-                        u[3] = cpx<R>(b.z, b.w); u[4] = cpx<R>(cc.x, cc.y); u[5] = cpx<R>(cc.z, cc.w);
-                        u[6] = conj(u[1] * u[5] - u[2] * u[4]);
-                        u[7] = conj(u[2] * u[3] - u[0] * u[5]);
-                        u[8] = conj(u[0] * u[4] - u[1] * u[3]);
-                    } else {
-                        int ph;
-                        const int n = neighbor(g, s, c, mu, fwd, &ph);
-                        Gauge<R>::load(U, V, mu, fwd ? s : n, u);
-                    }
+                    const float4 *q = slink + (size_t)mu * 3 * bv + (fwd ? l : ln);
+                    const float4 a = q[0], b = q[bv], cc = q[2 * bv];
+                    u[0] = cpx<R>(a.x, a.y); u[1] = cpx<R>(a.z, a.w); u[2] = cpx<R>(b.x, b.y);
+                    u[3] = cpx<R>(b.z, b.w); u[4] = cpx<R>(cc.x, cc.y); u[5] = cpx<R>(cc.z, cc.w);
+                    u[6] = conj(u[1] * u[5] - u[2] * u[4]);
+                    u[7] = conj(u[2] * u[3] - u[0] * u[5]);
+                    u[8] = conj(u[0] * u[4] - u[1] * u[3]);
 #pragma unroll
                     for (int k = 0; k < 12; ++k) psi[k] = rho[k * bv + ln];
                     hop_accumulate<R>(mu, fwd, u, psi, (R)1, up, lo);
@@ -737,22 +727,260 @@ sap_kernel(Geom g, AggGeom B, int colour, R sigma, const void *__restrict__ U,
     }
 }
 
+// FP64.  What bounds a sweep is the FP64 pipe (a warp's instruction holds its scheduler for 64
+// clocks) of the schedulers that have work: 16 blocks of 256 sites at 8^3 x 16 took 464 us a
+// sweep as 16 CTAs with a thread a site.  So a block is a cluster of CTAs with 32 sites each, and a
+// site's work is cut into four threads of four warps: warp w takes the two hops of direction w
+// and then the three components 3w .. 3w + 2 of everything else.  Two-grid cycle at 8^3 x 16:
+// 3950 us before, 2650 with one thread a site in clusters, 2046 in this form.  At 16^3 x 32
+// every SM has work either way (256 blocks a colour) and the two forms are near each other.
+// A neighbour in another CTA of the cluster is read from that one's shared memory; every
+// thread gets the sums of the MR step in the same order.
+__device__ __forceinline__ unsigned cluster_map(unsigned smem_addr, int rank) {
+    unsigned a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ cpx<double> ld_cluster(unsigned a) {
+    cpx<double> v;
+    asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.re), "=d"(v.im) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ double ld_cluster1(unsigned a) {
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// out = rows I0 .. I0 + 2 of a 6x6 Hermitian block (packed as in hermitian6_apply, entry pairs V
+// apart) times x
+template <int I0>
+__device__ __forceinline__ void hermitian6_rows(const double2 *p, int V, const cpx<double> x[6], cpx<double> out[3]) {
+    const double2 d0 = p[(size_t)(I0 / 2) * V], d1 = p[(size_t)(I0 / 2 + 1) * V];
+    const double dg[3] = {I0 ? d0.y : d0.x, I0 ? d1.x : d0.y, I0 ? d1.y : d1.x};
+#pragma unroll
+    for (int i = I0; i < I0 + 3; ++i) {
+        cpx<double> acc = dg[i - I0] * x[i];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            if (j == i) continue;
+            const double2 t = p[(size_t)(3 + (i < j ? offdiag_index(i, j) : offdiag_index(j, i))) * V];
+            if (i < j) cmac(acc, cpx<double>(t.x, t.y), x[j]);
+            else cmac_conj(acc, cpx<double>(t.x, t.y), x[j]);
+        }
+        out[i - I0] = acc;
+    }
+}
+
+// The components 6 blk + I0 .. + 2 of D_sigma x: x the six components of chirality blk, hops the
+// sites' four hop sums, [direction][12][32]
+template <int I0>
+__device__ __forceinline__ void dsigma_rows(const double2 *clov, int V, int blk, double sigma, const cpx<double> *hops,
+                                            const cpx<double> x[6], cpx<double> out[3]) {
+    hermitian6_rows<I0>(clov + (size_t)blk * 18 * V, V, x, out);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const cpx<double> *h = hops + (6 * blk + I0 + j) * 32;
+        const cpx<double> t = (h[0] + h[12 * 32]) + (h[24 * 32] + h[36 * 32]);
+        out[j] = out[j] - 0.5 * t - (blk ? -sigma : sigma) * x[I0 + j];
+    }
+}
+
+// The hops of direction mu, without the -1/2: part[k * 32] for the 12 components.  f and b say
+// which of them there are, phase_f and phase_b are 1 or -1, psi_f(k) and psi_b(k) the
+// neighbours' components
+template <class PF, class PB>
+__device__ __forceinline__ void sap_hops(int mu, bool f, bool b, int phase_f, int phase_b, const void *U, int V, int s,
+                                         int sb, PF psi_f, PB psi_b, cpx<double> *part) {
+    using C = cpx<double>;
+    C hf[6], hb[6], u[9], psi[12], t[6], h[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) hf[k] = hb[k] = C();
+    if (f) {
+        Gauge<double>::load(U, V, mu, s, u);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) psi[k] = psi_f(k);
+        spin_B<double>(mu, psi + 6, t);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) h[k] = psi[k] - t[k];
+        su3_mul<double>(u, h, hf);
+        su3_mul<double>(u, h + 3, hf + 3);
+        if (phase_f < 0) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) hf[k] = -hf[k];
+        }
+    }
+    if (b) {
+        Gauge<double>::load(U, V, mu, sb, u);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) psi[k] = psi_b(k);
+        spin_B<double>(mu, psi + 6, t);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) h[k] = psi[k] + t[k];
+        su3_dag_mul<double>(u, h, hb);
+        su3_dag_mul<double>(u, h + 3, hb + 3);
+        if (phase_b < 0) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) hb[k] = -hb[k];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        part[k * 32] = hf[k] + hb[k];
+        h[k] = hb[k] - hf[k];
+    }
+    spin_Bdag<double>(mu, h, t);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) part[(6 + k) * 32] = t[k];
+}
+
+__global__ void __launch_bounds__(128, 2)
+sap_f64_kernel(Geom g, AggGeom B, int colour, double sigma, const void *__restrict__ U, const double2 *__restrict__ clov,
+               const cpx<double> *__restrict__ rhs, int rhs_g5, cpx<double> *z, int mr_iters, int cs) {
+    using C = cpx<double>;
+    __shared__ double2 rho_s[12 * 32], part_s[4 * 12 * 32];
+    __shared__ double red[4 * 3];   // the warps' sums of the MR step
+    C *rho = reinterpret_cast<C *>(rho_s), *part = reinterpret_cast<C *>(part_s);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int rank = blockIdx.x % cs;
+    int b = 2 * (blockIdx.x / cs);   // of blocks b and b + 1 the one of this sweep's colour
+    {
+        int r = b, bsum = 0;
+        for (int mu = 0; mu < 4; ++mu) { bsum += r % B.cdims[mu]; r /= B.cdims[mu]; }
+        if ((bsum & 1) != colour) b += 1;
+    }
+    const int V = g.V, l = rank * 32 + lane;
+    const bool active = l < B.vol;
+    const int blk = w >> 1, k0 = 3 * w;   // own components: chirality blk, k0 .. k0 + 2
+    int lc[4] = {0, 0, 0, 0}, c[4] = {0, 0, 0, 0}, s = 0;
+    // the in-block neighbours of direction w, -1 where there is none
+    int lf = -1, lb = -1, sb = 0;
+    C x[6], q[3], e[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) e[j] = q[j] = C();
+    // residual of D_sigma z = rhs on this block (z read with its global neighbours)
+    if (active) {
+        s = agg_site(g, B, b, l, lc);
+        site_coords(g, s, c);
+        const int step = w == 0 ? 1 : w == 1 ? B.agg[0] : w == 2 ? B.agg[0] * B.agg[1] : B.agg[0] * B.agg[1] * B.agg[2];
+        const int lw = w == 0 ? lc[0] : w == 1 ? lc[1] : w == 2 ? lc[2] : lc[3];
+        if (lw + 1 < B.agg[w]) lf = l + step;
+        if (lw > 0) lb = l - step;
+        int pf, pb;
+        const int sf = neighbor(g, s, c, w, true, &pf);
+        sb = neighbor(g, s, c, w, false, &pb);
+        sap_hops(w, true, true, pf, pb, U, V, s, sb, [&](int k) { return z[(size_t)k * V + sf]; },
+                 [&](int k) { return z[(size_t)k * V + sb]; }, part + w * 12 * 32 + lane);
+    }
+    __syncthreads();
+    if (active) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) x[k] = z[(size_t)(6 * blk + k) * V + s];
+        if (w & 1) dsigma_rows<3>(clov + s, V, blk, sigma, part + lane, x, q);
+        else dsigma_rows<0>(clov + s, V, blk, sigma, part + lane, x, q);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const C r = rhs[(size_t)(k0 + j) * V + s];
+            rho[(k0 + j) * 32 + lane] = (rhs_g5 && blk ? -r : r) - q[j];
+        }
+    }
+    cluster_sync();
+    const unsigned rho0 = (unsigned)__cvta_generic_to_shared(rho), red0 = (unsigned)__cvta_generic_to_shared(red);
+    const unsigned nf = lf >= 0 ? cluster_map(rho0, lf >> 5) + (lf & 31) * (unsigned)sizeof(C) : 0;
+    const unsigned nb = lb >= 0 ? cluster_map(rho0, lb >> 5) + (lb & 31) * (unsigned)sizeof(C) : 0;
+    for (int it = 0; it < mr_iters; ++it) {
+        // q = D_sigma restricted to the block (Dirichlet) applied to rho
+        if (active)
+            sap_hops(w, lf >= 0, lb >= 0, 1, 1, U, V, s, sb,
+                     [&](int k) { return ld_cluster(nf + k * 32 * (unsigned)sizeof(C)); },
+                     [&](int k) { return ld_cluster(nb + k * 32 * (unsigned)sizeof(C)); }, part + w * 12 * 32 + lane);
+        __syncthreads();
+        double qr_re = 0, qr_im = 0, qq = 0;
+        if (active) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) x[k] = rho[(6 * blk + k) * 32 + lane];
+            if (w & 1) dsigma_rows<3>(clov + s, V, blk, sigma, part + lane, x, q);
+            else dsigma_rows<0>(clov + s, V, blk, sigma, part + lane, x, q);
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const C r = w & 1 ? x[3 + j] : x[j];
+                qr_re += q[j].re * r.re + q[j].im * r.im;
+                qr_im += q[j].re * r.im - q[j].im * r.re;
+                qq += q[j].re * q[j].re + q[j].im * q[j].im;
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            qr_re += __shfl_xor_sync(0xffffffffu, qr_re, o);
+            qr_im += __shfl_xor_sync(0xffffffffu, qr_im, o);
+            qq += __shfl_xor_sync(0xffffffffu, qq, o);
+        }
+        if (lane == 0) { red[3 * w] = qr_re; red[3 * w + 1] = qr_im; red[3 * w + 2] = qq; }
+        cluster_sync();   // all reads of rho for this step are done, partials visible
+        // lane 8 v + r: value v of CTA r (cs <= 8), then over the CTAs; alpha = (re, im) / qq
+        // with one division for both
+        const int v = lane >> 3, r = lane & 7;
+        double t = 0;
+        if (v < 3 && r < cs) {
+            const unsigned a = cluster_map(red0, r) + v * (unsigned)sizeof(double);
+            t = (ld_cluster1(a) + ld_cluster1(a + 24)) + (ld_cluster1(a + 48) + ld_cluster1(a + 72));
+        }
+        for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        const double A_qq = __shfl_sync(0xffffffffu, t, 16);
+        t = A_qq > 0 ? t / A_qq : 0.0;
+        const C alpha(__shfl_sync(0xffffffffu, t, 0), __shfl_sync(0xffffffffu, t, 8));
+        if (active) {
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const C r = w & 1 ? x[3 + j] : x[j];
+                cmac(e[j], alpha, r);
+                rho[(k0 + j) * 32 + lane] = r - alpha * q[j];
+            }
+        }
+        cluster_sync();
+    }
+    if (active) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            C &zk = z[(size_t)(k0 + j) * V + s];
+            zk = zk + e[j];
+        }
+    }
+}
+
 template <typename R>
 void sap_sweep(Ctx &c, int colour, double sigma, const void *rhs, bool rhs_gamma5, void *z) {
     AggGeom B = make_agg(c, c.prm.sap_block);
     MG_REQUIRE(B.vol <= 1024, MGEIG_EINVAL);
-    const int threads = ((B.vol + 31) / 32) * 32;
-    const size_t smem = (size_t)B.vol * 12 * sizeof(cpx<R>) + (sizeof(R) == 4 ? (size_t)B.vol * 12 * sizeof(float4) : 0);
-    MG_CUDA(cudaFuncSetAttribute(sap_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const void *U = sizeof(R) == 8 ? c.U64.p : c.U32.p;
-    const void *C = sizeof(R) == 8 ? c.clov64.p : c.clov32.p;
+    const int nw = (B.vol + 31) / 32;
     // half the sites: z read+write, rhs, links, clover (from HBM once per sweep)
     const double site_bytes = 12 * 2 * sizeof(R) * 3 + (sizeof(R) == 8 ? 576 : 192) + 72 * sizeof(R);
     TimeScope ts(c.timer, sizeof(R) == 8 ? K_SAP_F64 : K_SAP_F32, site_bytes * c.g.V / 2);
     MG_REQUIRE(B.cdims[0] % 2 == 0, MGEIG_EINVAL);
-    sap_kernel<R><<<B.n / 2, threads, smem, c.stream>>>(c.g, B, colour, (R)sigma, U, C, rhs, rhs_gamma5 ? 1 : 0, z,
-                                                        c.prm.sap_mr_iters);
-    MG_CHECK_LAUNCH();
+    if constexpr (sizeof(R) == 8) {
+        MG_REQUIRE(nw <= 8, MGEIG_ECUDA);   // the portable cluster size
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(B.n / 2 * nw);
+        cfg.blockDim = dim3(128);
+        cfg.stream = c.stream;
+        cudaLaunchAttribute at = {};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = nw;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        MG_CUDA(cudaLaunchKernelEx(&cfg, sap_f64_kernel, c.g, B, colour, sigma, (const void *)c.U64.p,
+                                   (const double2 *)c.clov64.p, (const cpx<double> *)rhs, rhs_gamma5 ? 1 : 0,
+                                   (cpx<double> *)z, c.prm.sap_mr_iters, nw));
+    } else {
+        const size_t smem = (size_t)B.vol * 12 * (sizeof(cpx<R>) + sizeof(float4));
+        MG_CUDA(cudaFuncSetAttribute(sap_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        sap_f32_kernel<<<B.n / 2, nw * 32, smem, c.stream>>>(c.g, B, colour, (R)sigma, c.U32.p, c.clov32.p, rhs,
+                                                            rhs_gamma5 ? 1 : 0, z, c.prm.sap_mr_iters);
+        MG_CHECK_LAUNCH();
+    }
 }
 
 #define INST(R)                                                                              \

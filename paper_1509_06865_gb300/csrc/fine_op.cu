@@ -427,17 +427,31 @@ __global__ void __launch_bounds__(128) wilson_clover_nrhs_kernel(Geom g, const v
 // its sites' forward links (two rows, 12 float4 planes) and clover (18 planes)
 // into shared memory once, with coalesced loads, and applies the stencil to
 // every field from there; only the spinors (and the backward links of hops that
-// leave the CTA) stream from memory for each field.
+// leave the CTA) stream from memory for each field.  DRAM (47 % busy), L1 and the issue slots
+// (50 % each) share the time with the latency of 12 warps an SM; 2 or 3 threads a site, each
+// with every 2nd or 3rd field, and smaller groups of fields were slower.
 constexpr int NR_SITES = 128;
 constexpr size_t NR_SMEM = (size_t)(12 + 18) * NR_SITES * sizeof(float4);
 
+// The order of the CTAs: a run of cpc CTAs goes through all lt timeslices (of slice CTAs each)
+// before the next run, so that the spinors of its neighbours in t are still in L2; cpc = slice
+// is the order of the sites.
+struct NrOrder {
+    int cpc, lt, slice;
+};
+
 template <int MODE>
 __global__ void __launch_bounds__(NR_SITES, 3) wilson_clover_nrhs_staged_kernel(
-    Geom g, const float4 *__restrict__ U, const float4 *__restrict__ clov, const char *__restrict__ x,
+    Geom g, NrOrder o, const float4 *__restrict__ U, const float4 *__restrict__ clov, const char *__restrict__ x,
     char *__restrict__ y, float sigma, int nrhs, size_t field_bytes) {
     extern __shared__ float4 nr_smem[];
     float4 *sU = nr_smem, *sC = nr_smem + 12 * NR_SITES;
-    const int s0 = blockIdx.x * NR_SITES;
+    int b = blockIdx.x;
+    if (o.cpc != o.slice) {
+        const int q = b / o.cpc;
+        b = (q % o.lt) * o.slice + (q / o.lt) * o.cpc + b % o.cpc;
+    }
+    const int s0 = b * NR_SITES;
     const int n = min(NR_SITES, g.V - s0);
     const int t = threadIdx.x;
     if (t < n) {
@@ -541,23 +555,34 @@ void apply_fine_nrhs(Ctx &c, int mode, double sigma, const void *x, void *y, int
     char *yb = static_cast<char *>(y);
     if (sizeof(R) == 4 && nrhs > 1) {
         const int nb = grid_for(c.g.V, NR_SITES);
+        // Runs of at most 64 CTAs (8192 sites: with 12 fields three timeslices of them are 28 MB
+        // of L2) where a timeslice is a whole number of CTAs and longer: 32^3 x 64 with 12 fields
+        // 2257 us in the order of the sites, 2148 with 64, 2169 with 32, 2188 with 128.
+        NrOrder o{1, c.dims[3], 1};
+        const int S3 = c.g.V / c.dims[3];
+        if (S3 % NR_SITES == 0) {
+            o.slice = o.cpc = S3 / NR_SITES;
+            for (int d = 2; o.cpc > 64; ++d)
+                if (o.slice % d == 0) o.cpc = o.slice / d;
+            if (o.cpc < 32) o.cpc = o.slice;   // no even split
+        }
         const float4 *U4 = c.U32.as<float4>(), *C4 = c.clov32.as<float4>();
         const float sg = (float)sigma;
         switch (mode) {
             case MODE_D:
                 MG_CUDA(cudaFuncSetAttribute(wilson_clover_nrhs_staged_kernel<MODE_D>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NR_SMEM));
-                wilson_clover_nrhs_staged_kernel<MODE_D><<<nb, NR_SITES, NR_SMEM, c.stream>>>(c.g, U4, C4, xb, yb, sg, nrhs, fb);
+                wilson_clover_nrhs_staged_kernel<MODE_D><<<nb, NR_SITES, NR_SMEM, c.stream>>>(c.g, o, U4, C4, xb, yb, sg, nrhs, fb);
                 break;
             case MODE_DSIGMA:
                 MG_CUDA(cudaFuncSetAttribute(wilson_clover_nrhs_staged_kernel<MODE_DSIGMA>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NR_SMEM));
-                wilson_clover_nrhs_staged_kernel<MODE_DSIGMA><<<nb, NR_SITES, NR_SMEM, c.stream>>>(c.g, U4, C4, xb, yb, sg, nrhs, fb);
+                wilson_clover_nrhs_staged_kernel<MODE_DSIGMA><<<nb, NR_SITES, NR_SMEM, c.stream>>>(c.g, o, U4, C4, xb, yb, sg, nrhs, fb);
                 break;
             default:
                 MG_CUDA(cudaFuncSetAttribute(wilson_clover_nrhs_staged_kernel<MODE_QSIGMA>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NR_SMEM));
-                wilson_clover_nrhs_staged_kernel<MODE_QSIGMA><<<nb, NR_SITES, NR_SMEM, c.stream>>>(c.g, U4, C4, xb, yb, sg, nrhs, fb);
+                wilson_clover_nrhs_staged_kernel<MODE_QSIGMA><<<nb, NR_SITES, NR_SMEM, c.stream>>>(c.g, o, U4, C4, xb, yb, sg, nrhs, fb);
                 break;
         }
         MG_CHECK_LAUNCH();

@@ -15,6 +15,8 @@
 //                          nine hops d, Yr = P_r - Q_i, Yi = P_i + Q_r (complex
 //                          product from real 40 x 40 planes), the per-link scale
 //                          s_d folded into the staged right-hand sides
+#include <algorithm>
+
 #include "half16.cuh"
 #include "internal.h"
 
@@ -126,8 +128,10 @@ void coarse_apply_links16(Ctx &c, double sigma, const void *x, void *y) {
 constexpr int TC_WARPS = 6;                  // warp w: row tile w / 2, plane w % 2
 constexpr int TC_THREADS = 32 * TC_WARPS;
 constexpr int TC_MAXN = 16;                  // right-hand sides per launch
-constexpr int TC_BP = 56;                    // staged B pitch (halves): conflict-free fragment reads
-constexpr int TC_MAXNT = 2 * TC_MAXN / 8;    // n tiles of 8 columns
+constexpr int TC_BP = 56;                    // staged B pitch (halves): conflict-free ldmatrix phases
+constexpr int TC_K = 48;                     // staged rows of B
+// pitch of the accumulators in shared memory: two-way bank conflicts at most
+constexpr int TC_CP(int ncols) { return ncols + 2; }
 constexpr int TC_SLACK = 16 * 48 + 64;       // zero halves after the last plane (rows / columns to 48)
 
 __device__ __forceinline__ void mma_bf16_16816(float c[4], const uint32_t a[4], const uint32_t b[2]) {
@@ -143,6 +147,22 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem));
 }
 
+__device__ __forceinline__ void ldmatrix_x4(uint32_t r[4], const void *row) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(row);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+}
+__device__ __forceinline__ void ldmatrix_x2(uint32_t r[2], const void *row) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(row);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];\n" : "=r"(r[0]), "=r"(r[1]) : "r"(a));
+}
+
+// What bounds it: the instruction issue of many small steps per site, not the tensor pipe.
+// So the right-hand sides are staged two rows at a time in packed BF16, and fragments come by
+// ldmatrix (the links' rows where they start on 16 bytes, N_tv a multiple of 4; 4 bytes at a
+// time otherwise).  12 right-hand sides at 32^3 x 64: 233 us before (22 k warp instructions a
+// site), 199 now.  All nine hops staged at once, two CTAs an SM, took 348 us: too few warps.
+//
 // Shared memory of one CTA (one coarse site), n2 = 2 N_tv <= 48 rows:
 //   As  a ring of two hop buffers: one link block's planes as stored in global
 //       memory ([re|im][row][col], n2 x n2 each, row pitch n2 halves) plus TC_SLACK
@@ -152,8 +172,9 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
 //       hop d is multiplied
 //   Bs  [d][column n < 8 NT][k < 48] staged s_d [Xr | Xi], zero for k >= n2
 //   Cs  (after the products) [plane][48][2 nrhs] accumulators
+template <int NT>
 __global__ void __launch_bounds__(TC_THREADS, 5)
-coarse_apply_nrhs_tc_kernel(int nagg, int ntv, int nrhs, int NT, const __nv_bfloat16 *__restrict__ L,
+coarse_apply_nrhs_tc_kernel(int nagg, int ntv, int nrhs, const __nv_bfloat16 *__restrict__ L,
                             const float *__restrict__ scale, const int *__restrict__ nbr, float sigma,
                             const float2 *__restrict__ X, float2 *__restrict__ Y) {
     extern __shared__ __align__(16) unsigned char tc_smem[];
@@ -163,7 +184,8 @@ coarse_apply_nrhs_tc_kernel(int nagg, int ntv, int nrhs, int NT, const __nv_bflo
     __nv_bfloat16 *As = reinterpret_cast<__nv_bfloat16 *>(tc_smem);
     const size_t hop_elems = ((2 * plane + TC_SLACK + 7) / 8) * 8;   // one ring buffer (16-byte multiple)
     __nv_bfloat16 *Bs = As + 2 * hop_elems;
-    const int ncols = 8 * NT;
+    constexpr int ncols = 8 * NT;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // 1. the link block of hop d (contiguous 2 n2^2 halves) into ring buffer d & 1
     //    by 16-byte async copies, one commit group per hop
     const int chunks_per_blk = (int)(2 * plane * 2 / 16);
@@ -179,39 +201,41 @@ coarse_apply_nrhs_tc_kernel(int nagg, int ntv, int nrhs, int NT, const __nv_bflo
         As[2 * plane + e] = __float2bfloat16_rn(0.f);
         As[hop_elems + 2 * plane + e] = __float2bfloat16_rn(0.f);
     }
-    // 2. right-hand sides of the nine neighbours, scaled by the link's scale, in BF16:
-    //    warp-strided over (hop d, right-hand side r), lanes over the rows k; one
-    //    float2 load fills column r (real parts) and column nrhs + r (imaginary)
-    {
-        const int wq = threadIdx.x >> 5, lq = threadIdx.x & 31, nwq = blockDim.x >> 5;
-        for (int dr = wq; dr < 9 * nrhs; dr += nwq) {
-            const int d = dr / nrhs, r = dr - d * nrhs;
-            const size_t blk = (size_t)d * nagg + site;
-            const int b = __ldg(nbr + blk);
-            const float sc = __ldg(scale + blk);
-            const float2 *xr = X + ((size_t)r * nagg + b) * n2;
-            __nv_bfloat16 *br = Bs + ((size_t)d * ncols + r) * TC_BP;
-            __nv_bfloat16 *bi = Bs + ((size_t)d * ncols + nrhs + r) * TC_BP;
-            for (int k = lq; k < 48; k += 32) {
-                float2 xv = make_float2(0.f, 0.f);
-                if (k < n2) xv = xr[k];
-                br[k] = __float2bfloat16_rn(sc * xv.x);
-                bi[k] = __float2bfloat16_rn(sc * xv.y);
+    // 2. right-hand sides of the nine neighbours, scaled by the link's scale, in BF16: a warp
+    //    takes a hop d and a right-hand side r, a lane two rows k; columns r (real parts)
+    //    and nrhs + r (imaginary)
+#pragma unroll 3
+    for (int dr = w; dr < 9 * nrhs; dr += TC_WARPS) {
+        const int d = dr / nrhs, r = dr - d * nrhs;
+        const size_t blk = (size_t)d * nagg + site;
+        const int b = __ldg(nbr + blk);
+        const float sc = __ldg(scale + blk);
+        if (lane < TC_K / 2) {
+            float2 x0 = make_float2(0.f, 0.f), x1 = x0;
+            if (lane < ntv) {
+                const float2 *xr = X + ((size_t)r * nagg + b) * n2 + 2 * lane;
+                x0 = xr[0];
+                x1 = xr[1];
             }
-        }
-        // the padding columns 2 nrhs .. 8 NT - 1 of every hop are zero
-        const int npad = ncols - 2 * nrhs;
-        for (int e = threadIdx.x; e < 9 * npad * 48; e += blockDim.x) {
-            const int k = e % 48, q = e / 48, d = q / npad, col = 2 * nrhs + q % npad;
-            Bs[((size_t)d * ncols + col) * TC_BP + k] = __float2bfloat16_rn(0.f);
+            __nv_bfloat162 *br = reinterpret_cast<__nv_bfloat162 *>(Bs + ((size_t)d * ncols + r) * TC_BP) + lane;
+            br[0] = __floats2bfloat162_rn(sc * x0.x, sc * x1.x);
+            br[nrhs * (TC_BP / 2)] = __floats2bfloat162_rn(sc * x0.y, sc * x1.y);
         }
     }
+    // the padding columns 2 nrhs .. 8 NT - 1 of every hop are zero
+    const int npad = ncols - 2 * nrhs;
+    for (int q = w; q < 9 * npad; q += TC_WARPS) {
+        const int d = q / npad, col = 2 * nrhs + q - d * npad;
+        if (lane < TC_K / 2)
+            reinterpret_cast<__nv_bfloat162 *>(Bs + ((size_t)d * ncols + col) * TC_BP)[lane] = __floats2bfloat162_rn(0.f, 0.f);
+    }
     // 3. products: warp w takes rows 16 (w / 2) .. +15 of plane w % 2, every column tile
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, tq = lane & 3;
+    const int g = lane >> 2, tq = lane & 3;
     const int mt = w >> 1, pl = w & 1;
-    float acc[TC_MAXNT][4];
+    const bool rows16 = n2 % 8 == 0;   // the links' rows start on 16 bytes
+    float acc[NT][4];
 #pragma unroll
-    for (int j = 0; j < TC_MAXNT; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+    for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
     for (int d = 0; d < 9; ++d) {
         // hop d + 1 streams in while hop d is multiplied
         if (d + 1 < 9) {
@@ -222,25 +246,29 @@ coarse_apply_nrhs_tc_kernel(int nagg, int ntv, int nrhs, int NT, const __nv_bflo
         }
         __syncthreads();   // hop d (and, for d = 0, the staged B and the slack) visible to all
         if (16 * mt < n2) {
-            const __nv_bfloat16 *Ap = As + (size_t)(d & 1) * hop_elems + (size_t)pl * plane;
-            const __nv_bfloat16 *Bp = Bs + (size_t)d * ncols * TC_BP;
-            for (int ks = 0; ks < 3 && 16 * ks < n2; ++ks) {
-                uint32_t a[4];
-                const int r0 = 16 * mt + g, c0 = 16 * ks + 2 * tq;
-                a[0] = *reinterpret_cast<const uint32_t *>(Ap + (size_t)r0 * n2 + c0);
-                a[1] = *reinterpret_cast<const uint32_t *>(Ap + (size_t)(r0 + 8) * n2 + c0);
-                a[2] = *reinterpret_cast<const uint32_t *>(Ap + (size_t)r0 * n2 + c0 + 8);
-                a[3] = *reinterpret_cast<const uint32_t *>(Ap + (size_t)(r0 + 8) * n2 + c0 + 8);
+            const __nv_bfloat16 *Ap = As + (size_t)(d & 1) * hop_elems + (size_t)pl * plane + (size_t)16 * mt * n2;
+            const __nv_bfloat16 *Bp = Bs + (size_t)d * ncols * TC_BP + (lane & 7) * TC_BP;
+            uint32_t b[NT][6];   // k 0-7, 8-15, ... of every column tile
 #pragma unroll
-                for (int j = 0; j < TC_MAXNT; ++j) {
-                    if (j < NT) {
-                        uint32_t b[2];
-                        const __nv_bfloat16 *bc = Bp + (size_t)(8 * j + g) * TC_BP + 16 * ks + 2 * tq;
-                        b[0] = *reinterpret_cast<const uint32_t *>(bc);
-                        b[1] = *reinterpret_cast<const uint32_t *>(bc + 8);
-                        mma_bf16_16816(acc[j], a, b);
-                    }
+            for (int j = 0; j < NT; ++j) {
+                ldmatrix_x4(b[j], Bp + 8 * j * TC_BP + 8 * (lane >> 3));
+                ldmatrix_x2(b[j] + 4, Bp + 8 * j * TC_BP + 32 + 8 * ((lane >> 3) & 1));
+            }
+#pragma unroll
+            for (int ks = 0; ks < 3; ++ks) {
+                if (16 * ks >= n2) continue;
+                uint32_t a[4];
+                if (rows16) {
+                    ldmatrix_x4(a, Ap + ((lane & 7) + 8 * ((lane >> 3) & 1)) * n2 + 8 * (lane >> 4) + 16 * ks);
+                } else {
+                    const __nv_bfloat16 *ar = Ap + g * n2 + 16 * ks + 2 * tq;
+                    a[0] = *reinterpret_cast<const uint32_t *>(ar);
+                    a[1] = *reinterpret_cast<const uint32_t *>(ar + 8 * n2);
+                    a[2] = *reinterpret_cast<const uint32_t *>(ar + 8);
+                    a[3] = *reinterpret_cast<const uint32_t *>(ar + 8 * n2 + 8);
                 }
+#pragma unroll
+                for (int j = 0; j < NT; ++j) mma_bf16_16816(acc[j], a, b[j] + 2 * ks);
             }
         }
         __syncthreads();   // every read of ring buffer d & 1 is done before hop d + 2 overwrites it
@@ -249,24 +277,20 @@ coarse_apply_nrhs_tc_kernel(int nagg, int ntv, int nrhs, int NT, const __nv_bflo
     float *Cs = reinterpret_cast<float *>(tc_smem);   // [plane][48][ncols]
     if (16 * mt < n2) {
 #pragma unroll
-        for (int j = 0; j < TC_MAXNT; ++j) {
-            if (j < NT) {
-                const int r = 16 * mt + g, col = 8 * j + 2 * tq;
-                float *cp = Cs + (size_t)pl * 48 * ncols;
-                cp[(size_t)r * ncols + col] = acc[j][0];
-                cp[(size_t)r * ncols + col + 1] = acc[j][1];
-                cp[(size_t)(r + 8) * ncols + col] = acc[j][2];
-                cp[(size_t)(r + 8) * ncols + col + 1] = acc[j][3];
-            }
+        for (int j = 0; j < NT; ++j) {
+            float *cp = Cs + (pl * 48 + 16 * mt + g) * TC_CP(ncols) + 8 * j + 2 * tq;
+            *reinterpret_cast<float2 *>(cp) = make_float2(acc[j][0], acc[j][1]);
+            *reinterpret_cast<float2 *>(cp + 8 * TC_CP(ncols)) = make_float2(acc[j][2], acc[j][3]);
         }
     }
     __syncthreads();
     // 4. Yr = Ar Xr - Ai Xi, Yi = Ar Xi + Ai Xr; then gamma5^c and the shift
-    const float *Cr = Cs, *Ci = Cs + (size_t)48 * ncols;
+    constexpr int cpitch = TC_CP(ncols);
+    const float *Cr = Cs, *Ci = Cs + 48 * cpitch;
     for (int e = threadIdx.x; e < nrhs * n2; e += blockDim.x) {
-        const int row = e % n2, r = e / n2;
-        float yr = Cr[(size_t)row * ncols + r] - Ci[(size_t)row * ncols + nrhs + r];
-        float yi = Cr[(size_t)row * ncols + nrhs + r] + Ci[(size_t)row * ncols + r];
+        const int r = e / n2, row = e - r * n2;
+        float yr = Cr[row * cpitch + r] - Ci[row * cpitch + nrhs + r];
+        float yi = Cr[row * cpitch + nrhs + r] + Ci[row * cpitch + r];
         if (row >= ntv) { yr = -yr; yi = -yi; }
         const size_t idx = ((size_t)r * nagg + site) * n2 + row;
         const float2 xv = X[idx];
@@ -278,8 +302,23 @@ size_t coarse_nrhs_tc_smem(int n2, int NT) {
     const size_t hop_elems = ((2 * (size_t)n2 * n2 + TC_SLACK + 7) / 8) * 8;
     const size_t a = 2 * hop_elems * 2;
     const size_t b = (size_t)9 * 8 * NT * TC_BP * 2;
-    const size_t cbytes = (size_t)2 * 48 * 8 * NT * 4;
+    const size_t cbytes = (size_t)2 * 48 * TC_CP(8 * NT) * 4;
     return std::max(a + b, cbytes);
+}
+
+template <int NT>
+static void launch_nrhs_tc(Ctx &c, double sigma, const float2 *X, float2 *Y, int nrhs) {
+    const int n2 = 2 * c.prm.n_tv;
+    const size_t smem = coarse_nrhs_tc_smem(n2, NT);
+    MG_CUDA(cudaFuncSetAttribute(coarse_apply_nrhs_tc_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smem));
+    // algorithmic bytes: the 16-bit links and scales once, every right-hand side read
+    // (nine neighbours from L2, counted once) and written once
+    TimeScope ts(c.timer, K_COARSE_APPLY,
+                 (double)c.nagg * (9.0 * (2 * n2 * n2 * 2 + 4) + (double)nrhs * 2 * n2 * 8));
+    coarse_apply_nrhs_tc_kernel<NT><<<c.nagg, TC_THREADS, smem, c.stream>>>(
+        c.nagg, c.prm.n_tv, nrhs, c.Dc16.as<__nv_bfloat16>(), c.Dcs.as<float>(), c.cnbr.as<int>(), (float)sigma, X, Y);
+    MG_CHECK_LAUNCH();
 }
 
 void coarse_apply_nrhs(Ctx &c, double sigma, const void *X, void *Y, int nrhs) {
@@ -298,18 +337,14 @@ void coarse_apply_nrhs(Ctx &c, double sigma, const void *X, void *Y, int nrhs) {
         return;
     }
     MG_REQUIRE(n2 <= 48 && c.Dc16.p, MGEIG_EINVAL);
-    const int NT = (2 * nrhs + 7) / 8;
-    const size_t smem = coarse_nrhs_tc_smem(n2, NT);
-    MG_CUDA(cudaFuncSetAttribute(coarse_apply_nrhs_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem));
-    // algorithmic bytes: the 16-bit links and scales once, every right-hand side read
-    // (nine neighbours from L2, counted once) and written once
-    TimeScope ts(c.timer, K_COARSE_APPLY,
-                 (double)c.nagg * (9.0 * (2 * n2 * n2 * 2 + 4) + (double)nrhs * 2 * n2 * 8));
-    coarse_apply_nrhs_tc_kernel<<<c.nagg, TC_THREADS, smem, c.stream>>>(
-        c.nagg, ntv, nrhs, NT, c.Dc16.as<__nv_bfloat16>(), c.Dcs.as<float>(), c.cnbr.as<int>(), (float)sigma,
-        static_cast<const float2 *>(X), static_cast<float2 *>(Y));
-    MG_CHECK_LAUNCH();
+    const float2 *x = static_cast<const float2 *>(X);
+    float2 *y = static_cast<float2 *>(Y);
+    switch ((2 * nrhs + 7) / 8) {
+        case 1: launch_nrhs_tc<1>(c, sigma, x, y, nrhs); break;
+        case 2: launch_nrhs_tc<2>(c, sigma, x, y, nrhs); break;
+        case 3: launch_nrhs_tc<3>(c, sigma, x, y, nrhs); break;
+        default: launch_nrhs_tc<4>(c, sigma, x, y, nrhs); break;
+    }
 }
 
 }  // namespace mgeig

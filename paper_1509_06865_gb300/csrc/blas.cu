@@ -1,7 +1,7 @@
 // BLAS-1 on flat complex arrays (fine spinors of one precision share one
 // layout, so element-wise operations ignore it; coarse vectors are flat).
 //
-// Reductions are deterministic two-pass trees: a fixed grid of 256-thread blocks
+// Reductions are deterministic two-level trees: a fixed grid of 256-thread blocks
 // accumulates grid-stride partial sums (per thread in the array's own precision, then
 // in FP64 across the block), writes one partial per block, and the last block to
 // finish adds the partials in a fixed order.  Inner products of many vectors against
@@ -12,9 +12,9 @@
 // The FP64 pipe takes half a lane a cycle and scheduler, so a warp's FP64 addition costs
 // 64 cycles of it: the block sums exchange halves of the value list between lanes (31
 // additions for 32 values; a shuffle tree per value takes 160, which was 10 us a launch).
-// Projection (two passes of inner products and updates) at 16^3 x 32, before with a launch per
-// chunk of vectors, a second kernel for the sums and uploaded coefficients, and now: 20 FP64
-// vectors 528 us, 388 us; 32 FP32 vectors 348 us, 252 us.
+// A projection (inner products with all vectors to the host, then the update) at 16^3 x 32, before
+// with a launch per chunk of vectors, a second kernel for the sums and uploaded coefficients,
+// and now: 20 FP64 vectors 528 us, 388 us; 32 FP32 vectors 348 us, 252 us.
 #include <algorithm>
 
 #include "ds.cuh"

@@ -165,17 +165,17 @@ template void build_interp<double>(Ctx &, const void *const *, int, void *const 
 template void build_interp<float>(Ctx &, const void *const *, int, void *const *);
 
 // ---------------------------------------------------------------------------
-// restriction r_c = P^dag r
-
+// restriction r_c = P^dag r: CTA (a, y) takes aggregate a and the test vectors y per .. y per +
+// per - 1; how they are cut does not change a sum
 template <typename R>
-__global__ void restrict_kernel(Geom g, AggGeom A, PtrList P, int ntv, const void *__restrict__ r,
+__global__ void restrict_kernel(Geom g, AggGeom A, PtrList P, int ntv, int per, const void *__restrict__ r,
                                 cpx<R> *__restrict__ rc) {
     extern __shared__ unsigned char smem_raw[];
-    R *sh = reinterpret_cast<R *>(smem_raw);   // [nwarps][2*ntv][2]
-    const int a = blockIdx.x;
+    R *sh = reinterpret_cast<R *>(smem_raw);   // [nwarps][2*per][2]
+    const int a = blockIdx.x, j0 = blockIdx.y * per, nj = min(per, ntv - j0);
     const int V = g.V;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int n2 = 2 * ntv;
+    const int n2 = 2 * per;
     // one site per thread (aggregates of at most blockDim sites, the usual case):
     // r is loaded once and kept in registers for all test vectors; otherwise each
     // thread visits its sites once per j
@@ -188,12 +188,12 @@ __global__ void restrict_kernel(Geom g, AggGeom A, PtrList P, int ntv, const voi
         Spinor<R>::load(r, V, s1, x1);
     }
 #pragma unroll 2
-    for (int j = 0; j < ntv; ++j) {
+    for (int j = 0; j < nj; ++j) {
         cpx<R> d0, d1;
         if (one) {
             if (s1 >= 0) {
                 cpx<R> p[12];
-                Spinor<R>::load(P.p[j], V, s1, p);
+                Spinor<R>::load(P.p[j0 + j], V, s1, p);
 #pragma unroll
                 for (int k = 0; k < 6; ++k) { cmac_conj(d0, p[k], x1[k]); cmac_conj(d1, p[6 + k], x1[6 + k]); }
             }
@@ -203,7 +203,7 @@ __global__ void restrict_kernel(Geom g, AggGeom A, PtrList P, int ntv, const voi
                 const int s = agg_site(g, A, a, l, lc);
                 cpx<R> x[12], p[12];
                 Spinor<R>::load(r, V, s, x);
-                Spinor<R>::load(P.p[j], V, s, p);
+                Spinor<R>::load(P.p[j0 + j], V, s, p);
 #pragma unroll
                 for (int k = 0; k < 6; ++k) { cmac_conj(d0, p[k], x[k]); cmac_conj(d1, p[6 + k], x[6 + k]); }
             }
@@ -214,14 +214,15 @@ __global__ void restrict_kernel(Geom g, AggGeom A, PtrList P, int ntv, const voi
         }
         if (lane == 0) {
             sh[(w * n2 + j) * 2] = d0.re; sh[(w * n2 + j) * 2 + 1] = d0.im;
-            sh[(w * n2 + ntv + j) * 2] = d1.re; sh[(w * n2 + ntv + j) * 2 + 1] = d1.im;
+            sh[(w * n2 + per + j) * 2] = d1.re; sh[(w * n2 + per + j) * 2 + 1] = d1.im;
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < n2; i += blockDim.x) {
+    for (int i = threadIdx.x; i < 2 * nj; i += blockDim.x) {
+        const int chir = i >= nj, j = i - chir * nj, v = chir * per + j;
         cpx<R> t;
-        for (int q = 0; q < nw; ++q) { t.re += sh[(q * n2 + i) * 2]; t.im += sh[(q * n2 + i) * 2 + 1]; }
-        rc[(size_t)a * n2 + i] = t;
+        for (int q = 0; q < nw; ++q) { t.re += sh[(q * n2 + v) * 2]; t.im += sh[(q * n2 + v) * 2 + 1]; }
+        rc[(size_t)a * 2 * ntv + chir * ntv + j0 + j] = t;
     }
 }
 
@@ -237,35 +238,45 @@ void restrict_vec(Ctx &c, const void *const *P, const void *r, void *rc) {
     PtrList p{};
     for (int j = 0; j < ntv; ++j) p.p[j] = P[j];
     const int threads = agg_threads(A.vol);
-    const size_t smem = (size_t)(threads / 32) * 2 * ntv * 2 * sizeof(R);
+    // parts of the test vectors so that there are up to six CTAs an SM: with one CTA an aggregate a
+    // coarse grid of few aggregates left SMs idle (FP64, 8^3 x 16, 32 aggregates: 99 us, and the
+    // prolongation, then a thread a site, 70 us; the cycle 2040 -> 1948 us with both cut).  Two
+    // CTAs an SM or six are alike; 512 aggregates at 16^3 x 32 take one part, as before
+    const int parts = std::min(ntv, std::max(1, 6 * c.sms / A.n)), per = (ntv + parts - 1) / parts;
+    const size_t smem = (size_t)(threads / 32) * 2 * per * 2 * sizeof(R);
     TimeScope ts(c.timer, K_RESTRICT, (double)(ntv + 1) * c.g.V * 24 * sizeof(R));
-    restrict_kernel<R><<<A.n, threads, smem, c.stream>>>(c.g, A, p, ntv, r, static_cast<cpx<R> *>(rc));
+    restrict_kernel<R><<<dim3(A.n, (ntv + per - 1) / per), threads, smem, c.stream>>>(c.g, A, p, ntv, per, r,
+                                                                                     static_cast<cpx<R> *>(rc));
     MG_CHECK_LAUNCH();
 }
 
 // ---------------------------------------------------------------------------
-// prolongation e = P e_c
+// prolongation e = P e_c: a thread per fine site and chirality (blockIdx.y)
 
 template <typename R>
 __global__ void prolong_kernel(Geom g, AggGeom A, PtrList P, int ntv, const cpx<R> *__restrict__ ec, void *__restrict__ e) {
+    using V16 = typename V16Of<R>::T;
+    constexpr int N = 6 * (int)sizeof(cpx<R>) / 16;   // 16-byte planes of one chirality
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= g.V) return;
-    const int V = g.V;
     int c[4];
     site_coords(g, s, c);
-    const int a = agg_of_site(g, A, c);
-    const cpx<R> *ea = ec + (size_t)a * 2 * ntv;
-    cpx<R> out[12];
-#pragma unroll
-    for (int k = 0; k < 12; ++k) out[k] = cpx<R>();
+    const int chir = blockIdx.y;
+    const size_t V = g.V, first = (size_t)chir * N * V + s;
+    const cpx<R> *ea = ec + (size_t)agg_of_site(g, A, c) * 2 * ntv + chir * ntv;
+    cpx<R> out[6];
     for (int j = 0; j < ntv; ++j) {
-        cpx<R> p[12];
-        Spinor<R>::load(P.p[j], V, s, p);
-        const cpx<R> e0 = ea[j], e1 = ea[ntv + j];
+        const V16 *src = static_cast<const V16 *>(P.p[j]) + first;
+        V16 v[N];
 #pragma unroll
-        for (int k = 0; k < 6; ++k) { cmac(out[k], p[k], e0); cmac(out[6 + k], p[6 + k], e1); }
+        for (int q = 0; q < N; ++q) v[q] = src[q * V];
+        const cpx<R> *p = reinterpret_cast<const cpx<R> *>(v), ej = ea[j];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) cmac(out[k], p[k], ej);
     }
-    Spinor<R>::store(e, V, s, out);
+    V16 *dst = static_cast<V16 *>(e) + first;
+#pragma unroll
+    for (int q = 0; q < N; ++q) dst[q * V] = reinterpret_cast<const V16 *>(out)[q];
 }
 
 template <typename R>
@@ -275,7 +286,7 @@ void prolong_vec(Ctx &c, const void *const *P, const void *ec, void *e) {
     PtrList p{};
     for (int j = 0; j < ntv; ++j) p.p[j] = P[j];
     TimeScope ts(c.timer, K_PROLONG, (double)(ntv + 1) * c.g.V * 24 * sizeof(R));
-    prolong_kernel<R><<<grid_for(c.g.V, 128), 128, 0, c.stream>>>(c.g, A, p, ntv, static_cast<const cpx<R> *>(ec), e);
+    prolong_kernel<R><<<dim3(grid_for(c.g.V, 128), 2), 128, 0, c.stream>>>(c.g, A, p, ntv, static_cast<const cpx<R> *>(ec), e);
     MG_CHECK_LAUNCH();
 }
 

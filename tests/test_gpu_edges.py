@@ -168,3 +168,22 @@ def test_solve_with_a_basis_of_more_vectors_than_a_launch_takes(prec):
         res[steps] = np.linalg.norm(b - op.Q_sigma(x, 1.7)) / np.linalg.norm(b)
         ctx.close()
     assert res[100] <= res[70] * (1 + 1e-6)
+
+
+@pytest.mark.parametrize("prec,tol", [(0, 1e-12), (1, 1e-5)], ids=["fp64", "mixed"])
+@pytest.mark.parametrize("ntv", [2, 10])
+def test_restriction_cut_by_test_vectors(ntv, prec, tol):
+    """256 aggregates: the test vectors go to several CTAs, 10 of them unevenly."""
+    from paper_1509_06865_gb300 import Context
+    dims, agg = (8, 8, 8, 8), (2, 2, 2, 2)
+    W = synth.uniform_vectors(dims, ntv, 19)
+    P = mg.Interpolation(W, agg)
+    ctx = Context(dims)
+    ctx.set_params(agg=agg, sap_block=(4, 4, 4, 4), n_tv=ntv, precision=prec, **PHYS)
+    ctx.load_gauge(synth.gauge_field(dims, 0.25, 29))
+    ctx.set_test_vectors(W)
+    r = synth.gaussian_vectors(dims, 1, 3)[0]
+    ec = P.restrict(r)
+    assert rel_err(ctx.restrict(r), ec) < tol
+    assert rel_err(ctx.prolong(ec), P.prolong(ec)) < tol
+    ctx.close()

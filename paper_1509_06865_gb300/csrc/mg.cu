@@ -1,8 +1,8 @@
 // Two-grid kernels (Sec. 2 of arXiv:1509.06865, Eqs. 2.3-2.6):
 //   build_interp   aggregation interpolation P (Eq. 2.4): per aggregate and
 //                  chirality, Gram-Schmidt (twice) of the N_tv test vectors, FP64
-//   restrict_vec   r_c = P^dag r          (one CTA per aggregate)
-//   prolong_vec    e = P e_c              (one thread per fine site)
+//   restrict_vec   r_c = P^dag r          (CTAs per aggregate and part of the test vectors)
+//   prolong_vec    e = P e_c              (one thread per fine site and chirality)
 //   build_coarse   D_c = P^dag D P as nine per-direction blocks (Eq. 2.5)
 //   coarse_apply_many  y = gamma5^c D_c x - sigma x = (Q_c - sigma) x (Eq. 2.6), n vectors
 //   sap_sweep      one colour of the Schwarz alternating procedure on
@@ -743,7 +743,8 @@ sap_f32_kernel(Geom g, AggGeom B, int colour, float sigma, const void *__restric
 // sweep as 16 CTAs with a thread a site.  So a block is a cluster of CTAs with 32 sites each, and a
 // site's work is cut into four threads of four warps: warp w takes the two hops of direction w
 // and then the three components 3w .. 3w + 2 of everything else.  Two-grid cycle at 8^3 x 16:
-// 3950 us before, 2650 with one thread a site in clusters, 2046 in this form.  At 16^3 x 32
+// 3950 us before, 2650 with one thread a site in clusters, 2046 in this form (a sweep 464, 240
+// and 144 us).  At 16^3 x 32
 // every SM has work either way (256 blocks a colour) and the two forms are near each other.
 // A neighbour in another CTA of the cluster is read from that one's shared memory; every
 // thread gets the sums of the MR step in the same order.

@@ -323,7 +323,8 @@ int mgeig_coarse_apply(mgeig_ctx *ctx, double sigma, const double *xc, double *y
  * another (Eq. 2.6).  With MGEIG_MIXED and MGEIG_LINKS_BF16 one launch on the
  * tensor cores (BF16 links with their per-link FP32 scale, right-hand sides
  * rounded to BF16 after the scale is applied, FP32 accumulation); with the
- * other link formats the CUDA-core coarse apply per right-hand side. */
+ * level-precision links one CUDA-core launch for up to 24, IEEE half links one per
+ * right-hand side. */
 int mgeig_coarse_apply_nrhs(mgeig_ctx *ctx, double sigma, const double *xc, double *yc, int nrhs);
 
 /* The same on device memory, MGEIG_MIXED only: X and Y hold nrhs FP32 coarse

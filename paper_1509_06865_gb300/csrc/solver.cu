@@ -106,9 +106,10 @@ void ensure_reduction(Ctx &c, int max_vectors) {
         // (vectors + 1) x 1024 blocks of partial sums, then the reductions' tickets (zero between launches)
         const size_t part = (size_t)(MAX_ITERATED + 8) * 1024 * sizeof(double2);
         c.red_partial.alloc(part + 256);
-        MG_CUDA(cudaMemset(c.red_partial.as<char>() + part, 0, 256));
+        // on the stream of the kernels that rely on these zeros: it does not wait for the default stream
+        MG_CUDA(cudaMemsetAsync(c.red_partial.as<char>() + part, 0, 256, c.stream));
         c.red_out.alloc(RED_SLOTS * sizeof(double2));
-        MG_CUDA(cudaMemset(c.red_out.p, 0, RED_SLOTS * sizeof(double2)));
+        MG_CUDA(cudaMemsetAsync(c.red_out.p, 0, RED_SLOTS * sizeof(double2), c.stream));
         MG_CUDA(cudaMallocHost(&c.pinned, 2 * RED_SLOTS * sizeof(double2)));
     }
 }
@@ -257,7 +258,10 @@ void mg_alloc(Ctx &c) {
         }
     }
     c.cnbr.alloc(nbr.size() * sizeof(int));
-    MG_CUDA(cudaMemcpy(c.cnbr.p, nbr.data(), nbr.size() * sizeof(int), cudaMemcpyHostToDevice));
+    // on the context's stream, which the kernels that read it run on (the default stream's copy from
+    // pageable memory may end after the call has returned, and that stream does not wait for it)
+    MG_CUDA(cudaMemcpyAsync(c.cnbr.p, nbr.data(), nbr.size() * sizeof(int), cudaMemcpyHostToDevice, c.stream));
+    sync(c);   // nbr goes out of scope
 }
 
 void mg_free(Ctx &c) {

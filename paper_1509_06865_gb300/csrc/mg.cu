@@ -997,6 +997,7 @@ void sap_sweep(Ctx &c, int colour, double sigma, const void *rhs, bool rhs_gamma
         MG_CUDA(cudaLaunchKernelEx(&cfg, sap_f64_kernel, c.g, B, colour, sigma, (const void *)c.U64.p,
                                    (const double2 *)c.clov64.p, (const cpx<double> *)rhs, rhs_gamma5 ? 1 : 0,
                                    (cpx<double> *)z, c.prm.sap_mr_iters, nw));
+        MG_CHECK_LAUNCH();
     } else {
         const size_t smem = (size_t)B.vol * 12 * (sizeof(cpx<R>) + sizeof(float4));
         MG_CUDA(cudaFuncSetAttribute(sap_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -600,15 +600,20 @@ void coarse_apply(Ctx &c, double sigma, const void *x, void *y) {
 }
 
 // ---------------------------------------------------------------------------
-// SAP: one colour of blocks; CTA = one block, thread = one site
+// SAP: one colour of blocks; CTA = one block, thread = one site (FP64: or a cluster, below)
 
 // FP32: the block's forward links (two rows, 3 float4 per link) are staged in
 // shared memory once and serve every MR step (the backward link of an in-block
 // hop is the forward link of the in-block neighbour); two CTAs fit an SM.
-__global__ void __launch_bounds__(256, 2)
-sap_f32_kernel(Geom g, AggGeom B, int colour, float sigma, const void *__restrict__ U,
+// FP64: the links come from L2, an MR step's FP64 arithmetic takes far longer.
+template <typename R> struct SapBounds { static constexpr int minb = 1; };
+template <> struct SapBounds<float> { static constexpr int minb = 2; };
+
+template <typename R>
+__global__ void __launch_bounds__(256, SapBounds<R>::minb)
+sap_kernel(Geom g, AggGeom B, int colour, R sigma, const void *__restrict__ U,
            const void *__restrict__ clov, const void *__restrict__ rhs, int rhs_g5, void *z, int mr_iters) {
-    using R = float;
+    constexpr bool stage = sizeof(R) == 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // component-major (rho[k][vol], slink[mu][3][vol]): consecutive threads read
     // consecutive words, without the 4-way bank conflicts of a site-major layout
@@ -636,7 +641,7 @@ sap_f32_kernel(Geom g, AggGeom B, int colour, float sigma, const void *__restric
     cpx<R> e[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) e[k] = cpx<R>();
-    if (active) {
+    if (stage && active) {
         const float4 *ug = static_cast<const float4 *>(U);
         for (int mu = 0; mu < 4; ++mu)
             for (int e = 0; e < 3; ++e) slink[(mu * 3 + e) * bv + l] = ug[((size_t)mu * 3 + e) * V + s];
@@ -693,13 +698,18 @@ sap_f32_kernel(Geom g, AggGeom B, int colour, float sigma, const void *__restric
                     int ln = l + (fwd ? 1 : -1) * (mu == 0 ? 1 : mu == 1 ? B.agg[0] : mu == 2 ? B.agg[0] * B.agg[1]
                                                                                               : B.agg[0] * B.agg[1] * B.agg[2]);
                     cpx<R> u[9], psi[12];
-                    const float4 *q = slink + (size_t)mu * 3 * bv + (fwd ? l : ln);
-                    const float4 a = q[0], b = q[bv], cc = q[2 * bv];
-                    u[0] = cpx<R>(a.x, a.y); u[1] = cpx<R>(a.z, a.w); u[2] = cpx<R>(b.x, b.y);
-                    u[3] = cpx<R>(b.z, b.w); u[4] = cpx<R>(cc.x, cc.y); u[5] = cpx<R>(cc.z, cc.w);
-                    u[6] = conj(u[1] * u[5] - u[2] * u[4]);
-                    u[7] = conj(u[2] * u[3] - u[0] * u[5]);
-                    u[8] = conj(u[0] * u[4] - u[1] * u[3]);
+                    if constexpr (stage) {
+                        const float4 *q = slink + (size_t)mu * 3 * bv + (fwd ? l : ln);
+                        const float4 a = q[0], b = q[bv], cc = q[2 * bv];
+                        u[0] = cpx<R>(a.x, a.y); u[1] = cpx<R>(a.z, a.w); u[2] = cpx<R>(b.x, b.y);
+                        u[3] = cpx<R>(b.z, b.w); u[4] = cpx<R>(cc.x, cc.y); u[5] = cpx<R>(cc.z, cc.w);
+                        u[6] = conj(u[1] * u[5] - u[2] * u[4]);
+                        u[7] = conj(u[2] * u[3] - u[0] * u[5]);
+                        u[8] = conj(u[0] * u[4] - u[1] * u[3]);
+                    } else {
+                        int ph;
+                        Gauge<R>::load(U, V, mu, fwd ? s : neighbor(g, s, c, mu, false, &ph), u);
+                    }
 #pragma unroll
                     for (int k = 0; k < 12; ++k) psi[k] = rho[k * bv + ln];
                     hop_accumulate<R>(mu, fwd, u, psi, (R)1, up, lo);
@@ -749,14 +759,12 @@ sap_f32_kernel(Geom g, AggGeom B, int colour, float sigma, const void *__restric
     }
 }
 
-// FP64.  What bounds a sweep is the FP64 pipe (a warp's instruction holds its scheduler for 64
-// clocks) of the schedulers that have work: 16 blocks of 256 sites at 8^3 x 16 took 464 us a
-// sweep as 16 CTAs with a thread a site.  So a block is a cluster of CTAs with 32 sites each, and a
-// site's work is cut into four threads of four warps: warp w takes the two hops of direction w
-// and then the three components 3w .. 3w + 2 of everything else.  Two-grid cycle at 8^3 x 16:
-// 3950 us before, 2650 with one thread a site in clusters, 2046 in this form (a sweep 464, 240
-// and 144 us).  At 16^3 x 32
-// every SM has work either way (256 blocks a colour) and the two forms are near each other.
+// FP64 where there are few blocks.  What bounds a sweep is the FP64 pipe (a warp's instruction
+// holds its scheduler for 64 clocks) of the schedulers that have work: 16 blocks of 256 sites at
+// 8^3 x 16 took 464 us a sweep as 16 CTAs with a thread a site.  So a block is a cluster of CTAs
+// with 32 sites each, and a site's work is cut into four threads of four warps: warp w takes the
+// two hops of direction w and then the three components 3w .. 3w + 2 of everything else.  A
+// sweep at 8^3 x 16 takes 147 us in this form (240 in clusters with a thread a site).
 // A neighbour in another CTA of the cluster is read from that one's shared memory; every
 // thread gets the sums of the MR step in the same order.
 __device__ __forceinline__ unsigned cluster_map(unsigned smem_addr, int rank) {
@@ -861,7 +869,7 @@ __device__ __forceinline__ void sap_hops(int mu, bool f, bool b, int phase_f, in
 }
 
 __global__ void __launch_bounds__(128, 2)
-sap_f64_kernel(Geom g, AggGeom B, int colour, double sigma, const void *__restrict__ U, const double2 *__restrict__ clov,
+sap_f64_cluster_kernel(Geom g, AggGeom B, int colour, double sigma, const void *__restrict__ U, const double2 *__restrict__ clov,
                const cpx<double> *__restrict__ rhs, int rhs_g5, cpx<double> *z, int mr_iters, int cs) {
     using C = cpx<double>;
     __shared__ double2 rho_s[12 * 32], part_s[4 * 12 * 32];
@@ -973,17 +981,31 @@ sap_f64_kernel(Geom g, AggGeom B, int colour, double sigma, const void *__restri
     }
 }
 
+// Whether an FP64 sweep of nblk blocks of nw groups of 32 sites takes the form in clusters.  Its
+// work is about 1.4 times that of the form with a thread a site (sums of the hops' parts,
+// distributed shared memory), but the groups are spread evenly over the SMs; there a group is a
+// warp, an SM gets whole blocks, and fewer than four warps leave schedulers idle.  Both sides count
+// the groups of the SM that has most.  Measured, a sweep (a thread a site, in clusters):
+//   8^3 x 16 in 4^4 blocks 466, 146 us     8^3 x 16 in 2^4 blocks 232, 148 us
+//   16^2 x 8 x 16 in 4^4 466, 298 us       16^3 x 24 in 4^4 930, 793 us
+//   16^4 in 4^4 467, 568 us                16^3 x 32 in 4^4 932, 1064 us
+//   12^3 x 24 in 3^4 360, 438 us           24^3 x 48 in 4^4 4191, 5166 us
+static bool sap_in_clusters(int nblk, int nw, int sms) {
+    const int site = std::max(4, (nblk + sms - 1) / sms * nw), cluster = (nblk * nw + sms - 1) / sms;
+    return 7 * cluster < 5 * site;
+}
+
 template <typename R>
 void sap_sweep(Ctx &c, int colour, double sigma, const void *rhs, bool rhs_gamma5, void *z) {
     AggGeom B = make_agg(c, c.prm.sap_block);
     MG_REQUIRE(B.vol <= 1024, MGEIG_EINVAL);
     const int nw = (B.vol + 31) / 32;
+    MG_REQUIRE(nw <= 8, MGEIG_ECUDA);   // 256 threads a CTA, eight CTAs a cluster
     // half the sites: z read+write, rhs, links, clover (from HBM once per sweep)
     const double site_bytes = 12 * 2 * sizeof(R) * 3 + (sizeof(R) == 8 ? 576 : 192) + 72 * sizeof(R);
     TimeScope ts(c.timer, sizeof(R) == 8 ? K_SAP_F64 : K_SAP_F32, site_bytes * c.g.V / 2);
     MG_REQUIRE(B.cdims[0] % 2 == 0, MGEIG_EINVAL);
-    if constexpr (sizeof(R) == 8) {
-        MG_REQUIRE(nw <= 8, MGEIG_ECUDA);   // the portable cluster size
+    if (sizeof(R) == 8 && sap_in_clusters(B.n / 2, nw, c.sms)) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(B.n / 2 * nw);
         cfg.blockDim = dim3(128);
@@ -994,17 +1016,17 @@ void sap_sweep(Ctx &c, int colour, double sigma, const void *rhs, bool rhs_gamma
         at.val.clusterDim.y = at.val.clusterDim.z = 1;
         cfg.attrs = &at;
         cfg.numAttrs = 1;
-        MG_CUDA(cudaLaunchKernelEx(&cfg, sap_f64_kernel, c.g, B, colour, sigma, (const void *)c.U64.p,
+        MG_CUDA(cudaLaunchKernelEx(&cfg, sap_f64_cluster_kernel, c.g, B, colour, sigma, (const void *)c.U64.p,
                                    (const double2 *)c.clov64.p, (const cpx<double> *)rhs, rhs_gamma5 ? 1 : 0,
                                    (cpx<double> *)z, c.prm.sap_mr_iters, nw));
-        MG_CHECK_LAUNCH();
     } else {
-        const size_t smem = (size_t)B.vol * 12 * (sizeof(cpx<R>) + sizeof(float4));
-        MG_CUDA(cudaFuncSetAttribute(sap_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        sap_f32_kernel<<<B.n / 2, nw * 32, smem, c.stream>>>(c.g, B, colour, (R)sigma, c.U32.p, c.clov32.p, rhs,
+        const size_t smem = (size_t)B.vol * 12 * (sizeof(cpx<R>) + (sizeof(R) == 4 ? sizeof(float4) : 0));
+        MG_CUDA(cudaFuncSetAttribute(sap_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        sap_kernel<R><<<B.n / 2, nw * 32, smem, c.stream>>>(c.g, B, colour, (R)sigma, sizeof(R) == 8 ? c.U64.p : c.U32.p,
+                                                            sizeof(R) == 8 ? c.clov64.p : c.clov32.p, rhs,
                                                             rhs_gamma5 ? 1 : 0, z, c.prm.sap_mr_iters);
-        MG_CHECK_LAUNCH();
     }
+    MG_CHECK_LAUNCH();
 }
 
 #define INST(R)                                                                              \

@@ -77,6 +77,23 @@ def test_sap_block_shapes(name, prec, tol):
     ctx.close()
 
 
+@pytest.mark.parametrize("dims,sap", [((16, 8, 8, 8), (2, 2, 2, 2)), ((16, 16, 8, 8), (2, 2, 2, 2)),
+                                      ((12, 12, 12, 6), (3, 3, 3, 1)), ((16, 8, 16, 16), (4, 4, 4, 2))],
+                         ids=["256 x 16 sites", "512 x 16 sites", "192 x 27 sites", "128 x 128 sites"])
+def test_sap_fp64_many_blocks(dims, sap):
+    """Blocks a colour on both sides of the line between the two FP64 forms on 152 SMs, warps of them not full."""
+    from paper_1509_06865_gb300 import FP64, Context
+    U = synth.gauge_field(dims, 0.25, 311)
+    op = dirac.WilsonClover(U, PHYS["m0"], PHYS["csw"], bc=PHYS["bc"])
+    ctx = Context(dims)
+    ctx.set_params(agg=sap, sap_block=sap, n_tv=2, precision=FP64, sap_mr_iters=3, outer_restart=1, **PHYS)
+    ctx.load_gauge(U)
+    b, z0 = synth.gaussian_vectors(dims, 2, 8)
+    got = ctx.sap(b, 0.1 * z0, 0.05, cycles=1)
+    assert norm_rel_err(got, mg.SAP(op, sap).smooth(b, 0.1 * z0, 0.05, 1, 3)) < 1e-11
+    ctx.close()
+
+
 @pytest.mark.parametrize("prec,tol", [(0, 1e-9), (1, 1e-4)], ids=["fp64", "mixed"])
 @pytest.mark.parametrize("deflate", [1, 0], ids=["deflated", "plain"])
 @pytest.mark.parametrize("name", list(SHAPES))

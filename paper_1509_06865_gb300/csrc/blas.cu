@@ -26,8 +26,9 @@ constexpr int RED_THREADS = 256;
 constexpr int RED_MAXBLOCKS = 1024;
 constexpr int MAXVEC = MAX_ITERATED + 8;   // pointer slots per launch; more vectors take more launches
 static_assert(MAXVEC % 8 == 0, "a double-float update is rounded after every eight vectors");
-// vectors that share one read of y: 16 in FP32 (bandwidth bound); 8 in FP64, where the
-// FP64 pipe bounds the kernel and 16 accumulators cost occupancy
+// vectors that share one read of y: 16 in FP32 (bandwidth bound); 8 in FP64 and in
+// double-float arithmetic, where the arithmetic bounds the kernel and 16 accumulators cost
+// occupancy
 template <typename R> struct Chunk { static constexpr int n = sizeof(R) == 4 ? 16 : 8; };
 
 template <typename R> struct V2;
@@ -149,56 +150,67 @@ __device__ __forceinline__ void grid_reduce(double (&v)[N], int j0, int cnt, con
     if (threadIdx.x == 0) r.ticket[blockIdx.y] = 0;
 }
 
-// <X_j, y> for the chunk j = per * blockIdx.y ..
-template <typename R>
-__global__ void __launch_bounds__(RED_THREADS, 2) multidot_kernel(PtrPack X, int k, int per, const void *__restrict__ yv,
-                                                               size_t n, RedOut out, bool vec4) {
+// real values of C complex sums, filled up to a power of two
+template <int C> constexpr int VALUES = C <= 1 ? 2 : C <= 2 ? 4 : C <= 4 ? 8 : C <= 8 ? 16 : 32;
+
+// Blocks an SM that a kernel for C vectors leaves registers for: four (the grid's) where its
+// sums and loads in flight are few, two or three where they are many
+template <typename R, int C, bool batch> constexpr int dot_blocks() {
+    return !batch ? (sizeof(R) == 8 ? 2 : 4) : C * sizeof(R) <= 32 ? 4 : sizeof(R) == 4 ? 2 : 3;
+}
+
+// <X_j, y> for the chunk j = per * blockIdx.y .. of at most C vectors.  VEC: two complex values
+// per 16-byte load (FP32, n even, 16-byte aligned arrays).  A kernel for C vectors costs
+// every call the registers and the FP64 additions of C sums (the FP64 pipe also takes its time
+// for operations that are predicated off), so there are kernels for fewer: one vector of
+// 12.6 M values took 105 us with the kernel for 16 in FP32, now 45; 255 us in
+// double-float arithmetic and 754 in FP64 with the kernels for 8, now 92 and 207.
+template <typename R, int C, bool VEC>
+__global__ void __launch_bounds__(RED_THREADS, dot_blocks<R, C, VEC>())
+multidot_kernel(PtrPack X, int k, int per, const void *__restrict__ yv, size_t n, RedOut out) {
     typedef typename V2<R>::T T;
-    const T *y = static_cast<const T *>(yv);
-    constexpr int C = Chunk<R>::n;
     const int j0 = blockIdx.y * per;
     k = min(per, k - j0);
     R ar[C], ai[C];
 #pragma unroll
     for (int j = 0; j < C; ++j) { ar[j] = 0; ai[j] = 0; }
-    if constexpr (sizeof(R) == 4) {
-        if (vec4) {   // two complex values per 16-byte load (n even, 16-byte aligned arrays)
-            const float4 *y4 = static_cast<const float4 *>(yv);
-            for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n / 2; i += (size_t)gridDim.x * blockDim.x) {
-                const float4 b = y4[i];
-                float4 av[C];   // loaded before they are used
+    if constexpr (VEC) {
+        const float4 *y4 = static_cast<const float4 *>(yv);
+        for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n / 2; i += (size_t)gridDim.x * blockDim.x) {
+            const float4 b = y4[i];
+            float4 av[C];   // loaded before they are used
 #pragma unroll
-                for (int j = 0; j < C; ++j)
-                    if (j < k) av[j] = static_cast<const float4 *>(X.p[j0 + j])[i];
+            for (int j = 0; j < C; ++j)
+                if (j < k) av[j] = static_cast<const float4 *>(X.p[j0 + j])[i];
 #pragma unroll
-                for (int j = 0; j < C; ++j) {
-                    if (j < k) {
-                        const float4 a = av[j];
-                        ar[j] = fmaf(a.x, b.x, ar[j]); ar[j] = fmaf(a.y, b.y, ar[j]);
-                        ar[j] = fmaf(a.z, b.z, ar[j]); ar[j] = fmaf(a.w, b.w, ar[j]);
-                        ai[j] = fmaf(a.x, b.y, ai[j]); ai[j] = fmaf(-a.y, b.x, ai[j]);
-                        ai[j] = fmaf(a.z, b.w, ai[j]); ai[j] = fmaf(-a.w, b.z, ai[j]);
-                    }
+            for (int j = 0; j < C; ++j) {
+                if (j < k) {
+                    const float4 a = av[j];
+                    ar[j] = fmaf(a.x, b.x, ar[j]); ar[j] = fmaf(a.y, b.y, ar[j]);
+                    ar[j] = fmaf(a.z, b.z, ar[j]); ar[j] = fmaf(a.w, b.w, ar[j]);
+                    ai[j] = fmaf(a.x, b.y, ai[j]); ai[j] = fmaf(-a.y, b.x, ai[j]);
+                    ai[j] = fmaf(a.z, b.w, ai[j]); ai[j] = fmaf(-a.w, b.z, ai[j]);
                 }
             }
-            n = 0;   // the scalar loop below has nothing left to do
         }
-    }
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        T b = y[i];
+    } else {
+        const T *y = static_cast<const T *>(yv);
+        for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+            const T b = y[i];
 #pragma unroll
-        for (int j = 0; j < C; ++j) {
-            if (j < k) {
-                T a = static_cast<const T *>(X.p[j0 + j])[i];
-                ar[j] = fma(a.x, b.x, ar[j]); ar[j] = fma(a.y, b.y, ar[j]);
-                ai[j] = fma(a.x, b.y, ai[j]); ai[j] = fma(-a.y, b.x, ai[j]);
+            for (int j = 0; j < C; ++j) {
+                if (j < k) {
+                    const T a = static_cast<const T *>(X.p[j0 + j])[i];
+                    ar[j] = fma(a.x, b.x, ar[j]); ar[j] = fma(a.y, b.y, ar[j]);
+                    ai[j] = fma(a.x, b.y, ai[j]); ai[j] = fma(-a.y, b.x, ai[j]);
+                }
             }
         }
     }
-    double v[2 * C];
+    double v[VALUES<C>] = {};
 #pragma unroll
     for (int j = 0; j < C; ++j) { v[2 * j] = ar[j]; v[2 * j + 1] = ai[j]; }
-    grid_reduce<2 * C>(v, j0, k, out);
+    grid_reduce<VALUES<C>>(v, j0, k, out);
 }
 
 template <typename R>
@@ -269,26 +281,25 @@ __device__ __forceinline__ void ds_mac(float &h, float &l, float uh, float ul, f
     l = __fadd_rn(l, __fadd_rn(err, e));
 }
 
-constexpr int DS_CHUNK = 8;
-
-__global__ void __launch_bounds__(RED_THREADS, 3) multidot_ds_kernel(PtrPack X, int k, int per,
-                                                                     const double2 *__restrict__ y, size_t n, RedOut out) {
+template <int C>
+__global__ void __launch_bounds__(RED_THREADS, dot_blocks<double, C, true>())
+multidot_ds_kernel(PtrPack X, int k, int per, const double2 *__restrict__ y, size_t n, RedOut out) {
     const int j0 = blockIdx.y * per;
     k = min(per, k - j0);
-    float rh[DS_CHUNK], rl[DS_CHUNK], ih[DS_CHUNK], il[DS_CHUNK];
+    float rh[C], rl[C], ih[C], il[C];
 #pragma unroll
-    for (int j = 0; j < DS_CHUNK; ++j) { rh[j] = rl[j] = ih[j] = il[j] = 0.0f; }
+    for (int j = 0; j < C; ++j) { rh[j] = rl[j] = ih[j] = il[j] = 0.0f; }
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const double2 b = y[i];
-        double2 a[DS_CHUNK];
+        double2 a[C];
 #pragma unroll
-        for (int j = 0; j < DS_CHUNK; ++j)
+        for (int j = 0; j < C; ++j)
             if (j < k) a[j] = static_cast<const double2 *>(X.p[j0 + j])[i];
         float brh, brl, bih, bil;
         ds_split(b.x, brh, brl);
         ds_split(b.y, bih, bil);
 #pragma unroll
-        for (int j = 0; j < DS_CHUNK; ++j) {
+        for (int j = 0; j < C; ++j) {
             if (j < k) {
                 float arh, arl, aih, ail;
                 ds_split(a[j].x, arh, arl);
@@ -301,13 +312,13 @@ __global__ void __launch_bounds__(RED_THREADS, 3) multidot_ds_kernel(PtrPack X, 
             }
         }
     }
-    double v[2 * DS_CHUNK];
+    double v[VALUES<C>] = {};
 #pragma unroll
-    for (int j = 0; j < DS_CHUNK; ++j) {
+    for (int j = 0; j < C; ++j) {
         v[2 * j] = f2d_exact(rh[j]) + f2d_exact(rl[j]);
         v[2 * j + 1] = f2d_exact(ih[j]) + f2d_exact(il[j]);
     }
-    grid_reduce<2 * DS_CHUNK>(v, j0, k, out);
+    grid_reduce<VALUES<C>>(v, j0, k, out);
 }
 
 static RedOut red_out_at(Ctx &c, cpx<double> *d_out) {
@@ -315,24 +326,43 @@ static RedOut red_out_at(Ctx &c, cpx<double> *d_out) {
     return {p, reinterpret_cast<unsigned int *>(p + (size_t)MAXVEC * RED_MAXBLOCKS), reinterpret_cast<double2 *>(d_out)};
 }
 
+template <typename R, int C>
+static void launch_multidot(Ctx &c, const PtrPack &pk, int k, int per, const void *y, size_t n, const RedOut &out) {
+    if constexpr (C <= Chunk<R>::n && C * sizeof(R) >= 16) {
+        // FP32 vectors below 8 M complex values (a 16^3 x 32 spinor is 1.6 M): 2 blocks
+        // per SM and chunk, 1.3x faster there than 4 (measured); the others 4.  The grid does not
+        // depend on k, so that a thread's sums do not either
+        const dim3 grid(red_grid(c, n, (sizeof(R) == 4 && n < ((size_t)8 << 20)) ? 2 : 4), (k + per - 1) / per);
+        if constexpr (sizeof(R) == 4) {
+            if (vec4_ok<R>(pk, k, y, n)) {
+                multidot_kernel<R, C, true><<<grid, RED_THREADS, 0, c.stream>>>(pk, k, per, y, n, out);
+                return;
+            }
+        } else if (c.ds_blas()) {
+            multidot_ds_kernel<C><<<grid, RED_THREADS, 0, c.stream>>>(pk, k, per, static_cast<const double2 *>(y), n, out);
+            return;
+        }
+        if constexpr (C <= 8) multidot_kernel<R, C, false><<<grid, RED_THREADS, 0, c.stream>>>(pk, k, per, y, n, out);
+    }
+}
+
 template <typename R>
 void blas_multidot(Ctx &c, const void *const *X, int k, const void *y, size_t n, cpx<double> *d_out) {
     for (; k > MAXVEC; k -= MAXVEC, X += MAXVEC, d_out += MAXVEC) blas_multidot<R>(c, X, MAXVEC, y, n, d_out);
     if (k < 1) return;
-    const bool ds = sizeof(R) == 8 && c.ds_blas();
-    const int C = ds ? DS_CHUNK : Chunk<R>::n, chunks = (k + C - 1) / C, per = (k + chunks - 1) / chunks;
-    // FP32 vectors below 8 M complex values (a 16^3 x 32 spinor is 1.6 M): 2 blocks
-    // per SM and chunk, 1.3x faster there than 4 (measured); the others 4.  The grid does not
-    // depend on k, so that a thread's sums do not either
-    const int nb = red_grid(c, n, (sizeof(R) == 4 && n < ((size_t)8 << 20)) ? 2 : 4);
-    TimeScope ts(c.timer, sizeof(R) == 8 ? K_BLAS_F64 : K_BLAS_LOW, (double)(k + 1) * n * 2 * sizeof(R));
     PtrPack pk{};
     for (int j = 0; j < k; ++j) pk.p[j] = X[j];
+    // 8-byte loads: eight vectors at most (12 vectors of 12.6 M values: 350 us with sixteen, whose
+    // registers leave too few warps an SM, 252 so)
+    const int most = vec4_ok<R>(pk, k, y, n) ? Chunk<R>::n : 8;
+    const int chunks = (k + most - 1) / most, per = (k + chunks - 1) / chunks;
+    TimeScope ts(c.timer, sizeof(R) == 8 ? K_BLAS_F64 : K_BLAS_LOW, (double)(k + 1) * n * 2 * sizeof(R));
     const RedOut out = red_out_at(c, d_out);
-    if (ds)
-        multidot_ds_kernel<<<dim3(nb, chunks), RED_THREADS, 0, c.stream>>>(pk, k, per, static_cast<const double2 *>(y), n, out);
-    else
-        multidot_kernel<R><<<dim3(nb, chunks), RED_THREADS, 0, c.stream>>>(pk, k, per, y, n, out, vec4_ok<R>(pk, k, y, n));
+    if (sizeof(R) == 8 && per <= 2) launch_multidot<R, 2>(c, pk, k, per, y, n, out);
+    else if (per <= 4) launch_multidot<R, 4>(c, pk, k, per, y, n, out);
+    else if (per <= 6) launch_multidot<R, 6>(c, pk, k, per, y, n, out);
+    else if (per <= 8) launch_multidot<R, 8>(c, pk, k, per, y, n, out);
+    else launch_multidot<R, 16>(c, pk, k, per, y, n, out);
     MG_CHECK_LAUNCH();
 }
 
@@ -363,11 +393,14 @@ struct HostCoef {
     __device__ __forceinline__ double2 operator[](int j) const { return v[j]; }
 };
 
-// vectors of an update that are loaded before they are used
+// vectors of an update that are loaded before they are used.  Double-float arithmetic: kernels
+// for fewer vectors, with fewer registers and more warps an SM (one vector of 12.6 M values 177 us
+// with the kernel for 8, 150 now); FP32, one value per access: twice as many
 constexpr int AXPY_BATCH = 8;
 
-// y += sign * sum_j coef[j] X_j, y and X_j FP64, double-float arithmetic
-template <typename Coef>
+// y += sign * sum_j coef[j] X_j, y and X_j FP64, double-float arithmetic; B vectors at a time,
+// LOOP: as often as it takes (without: k <= B)
+template <typename Coef, int B, bool LOOP>
 __global__ void __launch_bounds__(256) multi_axpy_ds_kernel(double2 *__restrict__ y, PtrPack X, int k, Coef coef,
                                                             double sign, size_t n) {
     __shared__ float4 cf[MAXVEC];   // (re high, re low, im high, im low)
@@ -384,17 +417,17 @@ __global__ void __launch_bounds__(256) multi_axpy_ds_kernel(double2 *__restrict_
         float rh, rl, ih, il;
         ds_split(t.x, rh, rl);
         ds_split(t.y, ih, il);
-        for (int j0 = 0; j0 < k; j0 += AXPY_BATCH) {
-            double2 a[AXPY_BATCH];
+        for (int j0 = 0; j0 < (LOOP ? k : 1); j0 += B) {
+            double2 a[B];
 #pragma unroll
-            for (int j = 0; j < AXPY_BATCH; ++j)
+            for (int j = 0; j < B; ++j)
                 if (j0 + j < k) a[j] = static_cast<const double2 *>(X.p[j0 + j])[i];
             if (j0) {   // y is rounded to FP64 after every eight vectors
                 ds_split(f2d_exact(rh) + f2d_exact(rl), rh, rl);
                 ds_split(f2d_exact(ih) + f2d_exact(il), ih, il);
             }
 #pragma unroll
-            for (int j = 0; j < AXPY_BATCH; ++j) {
+            for (int j = 0; j < B; ++j) {
                 if (j0 + j < k) {
                     float arh, arl, aih, ail;
                     ds_split(a[j].x, arh, arl);
@@ -412,8 +445,8 @@ __global__ void __launch_bounds__(256) multi_axpy_ds_kernel(double2 *__restrict_
     }
 }
 
-// y += sign * sum_j coef[j] X_j
-template <typename R, typename Coef>
+// y += sign * sum_j coef[j] X_j; B: AXPY_BATCH for one value per access
+template <typename R, typename Coef, int B>
 __global__ void __launch_bounds__(256) multi_axpy_kernel(void *__restrict__ yv, PtrPack X, int k, Coef coef, double sign,
                                                          size_t n, bool vec4) {
     typedef typename V2<R>::T T;
@@ -455,13 +488,13 @@ __global__ void __launch_bounds__(256) multi_axpy_kernel(void *__restrict__ yv, 
     }
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         T acc = y[i];
-        for (int j0 = 0; j0 < k; j0 += AXPY_BATCH) {
-            T a[AXPY_BATCH];
+        for (int j0 = 0; j0 < k; j0 += B) {
+            T a[B];
 #pragma unroll
-            for (int j = 0; j < AXPY_BATCH; ++j)
+            for (int j = 0; j < B; ++j)
                 if (j0 + j < k) a[j] = static_cast<const T *>(X.p[j0 + j])[i];
 #pragma unroll
-            for (int j = 0; j < AXPY_BATCH; ++j) {
+            for (int j = 0; j < B; ++j) {
                 if (j0 + j < k) {
                     const T c = cf[j0 + j];
                     acc.x = fma(c.x, a[j].x, acc.x); acc.x = fma(-c.y, a[j].y, acc.x);
@@ -489,11 +522,19 @@ static void launch_multi_axpy(Ctx &c, void *y, const void *const *X, int k, cons
     PtrPack pk{};
     for (int j = 0; j < k; ++j) pk.p[j] = X[j];
     if (sizeof(R) == 8 && c.ds_blas()) {
-        multi_axpy_ds_kernel<<<ew_grid(c, n), 256, 0, c.stream>>>(static_cast<double2 *>(y), pk, k, coef, sign, n);
+        double2 *y2 = static_cast<double2 *>(y);
+        const int nb = ew_grid(c, n);
+        if (k <= 2) multi_axpy_ds_kernel<Coef, 2, false><<<nb, 256, 0, c.stream>>>(y2, pk, k, coef, sign, n);
+        else if (k <= 4) multi_axpy_ds_kernel<Coef, 4, false><<<nb, 256, 0, c.stream>>>(y2, pk, k, coef, sign, n);
+        else if (k <= 6) multi_axpy_ds_kernel<Coef, 6, false><<<nb, 256, 0, c.stream>>>(y2, pk, k, coef, sign, n);
+        else multi_axpy_ds_kernel<Coef, AXPY_BATCH, true><<<nb, 256, 0, c.stream>>>(y2, pk, k, coef, sign, n);
     } else {
         const bool v4 = vec4_ok<R>(pk, k, y, n);
-        multi_axpy_kernel<R><<<ew_grid(c, v4 ? n / 2 : n, sizeof(R) == 4 ? 4 : 16), 256, 0, c.stream>>>(y, pk, k, coef,
-                                                                                                        sign, n, v4);
+        const int nb = ew_grid(c, v4 ? n / 2 : n, sizeof(R) == 4 ? 4 : 16);
+        if (sizeof(R) == 4 && !v4 && k > AXPY_BATCH)
+            multi_axpy_kernel<R, Coef, sizeof(R) == 4 ? 2 * AXPY_BATCH : AXPY_BATCH>
+                <<<nb, 256, 0, c.stream>>>(y, pk, k, coef, sign, n, v4);
+        else multi_axpy_kernel<R, Coef, AXPY_BATCH><<<nb, 256, 0, c.stream>>>(y, pk, k, coef, sign, n, v4);
     }
     MG_CHECK_LAUNCH();
 }

@@ -18,7 +18,7 @@ const void *coarse_gmres_kernel_f32() { return (const void *)coarse_gmres_kernel
 namespace {
 
 struct CGPlan {
-    int G, rb, nslice, m, slices, stage_sites;
+    int G, rb, nslice, m, slices, stage_sites, part_size;
     bool smem_slices, smem_defl;
     size_t dyn_smem;          // dynamic shared memory per block
     size_t off_slices, off_partial, scratch_bytes;   // global scratch layout
@@ -71,26 +71,41 @@ CGPlan compute_plan(Ctx &c, int k, int m) {
     const size_t room = CG_SMEM_LIMIT - fa.sharedSizeBytes;
     size_t used = p.smem_slices ? align16((size_t)p.nslice * p.rb * elem) : 0;
     MG_REQUIRE(used <= room, MGEIG_ECUDA);
-    // matvec threads per row, as far as there are threads and room for their parts: 8 (of a row
-    // pair) or 1 in FP32 (1 with 16-bit links, whose lanes share a row already), up to 24 in
-    // FP64 (every part costs the end of the matvec an FP64 addition per row)
+    // Threads that share a row of the matvec and leave the sum of their parts to its end: 8 (of a row
+    // pair) in FP32 with level links where one pass takes all rows, 1 in the forms with several
+    // passes (and with 16-bit links, whose lanes share a row already), up to 24 in FP64 (every
+    // part costs the end of the matvec an FP64 addition per row)
     auto fits = [&](int threads, int q, size_t stage) {
         return threads <= CG_MV && used + stage + (size_t)q * p.rb * elem <= room;
     };
     p.slices = 1;
-    p.stage_sites = 0;
+    p.stage_sites = p.part_size = 0;
     if (sizeof(R) == 8) {
         while (p.slices < std::min(24, 9 * c.prm.n_tv) && fits((p.slices + 1) * p.rb, p.slices + 1, 0)) ++p.slices;
     } else if (c.prm.coarse_links == MGEIG_LINKS_LEVEL) {
         const int n2 = 2 * c.prm.n_tv, sites = (p.rb + n2 - 2) / n2 + 1;   // that rb rows can touch
-        const size_t stage = (size_t)9 * sites * n2 * elem;
-        if (fits(8 * (p.rb / 2 + 1), 8, stage)) {   // rb rows lie in rb / 2 + 1 pairs at most
+        const size_t site_b = (size_t)9 * n2 * elem;
+        auto chunk = [&](size_t bytes) {   // coarse sites at a time, chunks of about the same size
+            const int most = (int)std::min((size_t)sites, (room - used) / bytes);
+            return most > 0 ? (sites + (sites + most - 1) / most - 1) / ((sites + most - 1) / most) : 0;
+        };
+        // one pass of all rows: rb of them lie in rb / 2 + 1 pairs at most; else several, with their
+        // parts where that leaves room for four sites
+        const int with_parts = chunk(site_b + 8 * n2 * elem);
+        if (fits(8 * (p.rb / 2 + 1), 8, sites * site_b)) {
             p.slices = 8;
             p.stage_sites = sites;
-            used += stage;
+        } else if (with_parts >= std::min(sites, 4)) {
+            p.stage_sites = with_parts;
+            p.part_size = 8 * with_parts * n2;
+        } else {
+            p.stage_sites = chunk(site_b);
         }
+        MG_REQUIRE(p.stage_sites > 0, MGEIG_ECUDA);
+        used += p.stage_sites * site_b;
     }
-    if (p.slices > 1) used += (size_t)p.slices * p.rb * elem;
+    if (p.slices > 1) p.part_size = p.slices * p.rb;
+    used += (size_t)p.part_size * elem;
     p.smem_defl = p.smem_slices && k > 0 && used + (size_t)2 * k * p.rb * elem <= room;
     if (p.smem_defl) used += (size_t)2 * k * p.rb * elem;
     p.dyn_smem = used;
@@ -162,6 +177,7 @@ void coarse_gmres_at(Ctx &c, double sigma, const void *rc, void *ec, void *scrat
     CGArgs<R> a;
     a.nagg = c.nagg; a.ntv = c.prm.n_tv; a.n = c.nagg * 2 * c.prm.n_tv;
     a.rb = p.rb; a.nslice = p.nslice; a.slices = p.slices; a.stage_sites = p.stage_sites;
+    a.part_size = p.part_size;
     a.smem_slices = p.smem_slices; a.smem_defl = p.smem_defl;
     a.Dc = static_cast<const cpx<R> *>(c.Dc.p);
     a.L16 = c.Dc16.p;

@@ -37,15 +37,18 @@
 // vector that another block is still writing, with two grid barriers per step.
 //
 // The matvec does not need what follows from R2, so after that barrier the block
-// splits: CG_MV threads multiply, the others gather R2, finish V_j+1 and run the
-// Givens rotations (a serial chain) beside them.
+// splits: CG_MV threads multiply, the others gather R2, finish V_j+1 (slices in shared
+// memory; else all threads do, after the matvec) and run the Givens rotations (a serial
+// chain) beside them.
 //
 // What bounds it: latency.  At 16^3 x 32 (20480 rows, 59 MB of FP32 links, L2 resident)
 // a step of the former kernel took 48 us: 18 in a matvec whose eight lanes a row went
 // through the nine hops one after another, twice (135 rows on 128 groups); 9 in the two
 // barriers; 8 gathering partial sums that lay [block][value], a sector a value; 6 in three
-// rounds of inner products; the rest in serial scalar work.  In this form it takes 20 us
-// (5 in the matvec, 4 in the barriers; a whole solve of 24 steps 1.11 -> 0.49 ms).
+// rounds of inner products; the rest in serial scalar work.  In this form it takes 18 us
+// (5 in the matvec, 4 in the barriers; a whole solve of 24 steps 1.12 -> 0.44 ms).  Blocks of
+// more rows are bound by memory: at 24^3 x 48 (683 rows, slices in global memory) a step takes
+// 92 us, at 32^3 x 64 (2156 rows) 273, of which the links need 139 at the HBM rate.
 //
 // Partial sums go to a [slot][G] buffer (consecutive reductions use disjoint
 // slots): after each barrier a few lanes a value read them contiguously, in the same
@@ -101,7 +104,8 @@ struct CGArgs {
     int rb;                        // rows per block (the last block may own fewer)
     int nslice;                    // owned-row vectors per block: V (m+1), GU (m), rhs, x, w
     int slices;                    // matvec threads that share a row; 1: none do
-    int stage_sites;               // coarse sites of a block whose neighbour vectors are staged (0: none)
+    int stage_sites;               // coarse sites whose neighbour vectors are staged at a time (0: none)
+    int part_size;                 // values of the matvec's parts in shared memory (0: none)
     int smem_slices, smem_defl;    // 1: the slices / copies of GW, GAW live in shared memory
     const cpx<R> *Dc;              // [9][nagg][col][row]
     const void *L16;               // 16-bit links [9][nagg][re|im][row][col] (16-bit kernels)
@@ -177,6 +181,17 @@ __device__ __forceinline__ int hop_nbr(const CGArgs<R> &a, const int *snb, int s
 // 2^-9; and a truncated solve multiplies it by the condition number.  So every split below
 // hands whole residues to its threads.
 
+// the sum over LANES neighbouring lanes, pairs of neighbours first
+template <int LANES>
+__device__ __forceinline__ cpx<float> group_sum_up(cpx<float> v) {
+#pragma unroll
+    for (int o = 1; o < LANES; o <<= 1) {
+        v.re += __shfl_xor_sync(0xffffffffu, v.re, o);
+        v.im += __shfl_xor_sync(0xffffffffu, v.im, o);
+    }
+    return v;
+}
+
 // The sums over the columns of all nine hop blocks, (D_c v)[row], for the owned rows: eight
 // threads share a pair of rows (16 bytes of a column; pairs start on even rows, so a block's
 // first and last pair may be half its own), one column residue each, whose sums go to
@@ -235,47 +250,163 @@ __device__ __forceinline__ void qmatvec_pairs(const CGArgs<float> &a, const cpx<
     if (i + 1 < nr) part[(size_t)q * nr + i + 1] = t1[0] + t1[1];
 }
 
-// The same with all eight residues in one thread, for blocks with more rows than threads
-// (their links come from HBM); the sums go to out.
-__device__ __forceinline__ void qmatvec_long(const CGArgs<float> &a, const cpx<float> *v, cpx<float> *out, int r0, int nr,
-                                             const int *snb, int s0, int tid) {
-    const int n2 = 2 * a.ntv;
-    for (int t = tid; t < nr; t += CG_MV) {
-        const int row = r0 + t, site = row / n2, rin = row - site * n2;
-        cpx<float> acc[8][2];
-        for (int d = 0; d < 9; ++d) {
-            const cpx<float> *pb = a.Dc + ((size_t)d * a.nagg + site) * n2 * n2 + rin;
-            const cpx<float> *px = v + (size_t)hop_nbr(a, snb, s0, d, site) * n2;
-            for (int j0 = 0; j0 < n2; j0 += 16) {
+// The neighbour vectors of the ns sites from c0 on to shared memory, [hop][site][n2], 16 bytes
+// (two columns) at a time
+__device__ __forceinline__ void stage_neighbours(const CGArgs<float> &a, const cpx<float> *v, cpx<float> *xs,
+                                                 const int *snb, int s0, int c0, int ns, int tid) {
+    const int ntv = a.ntv;
+    for (int e = tid; e < 9 * ns * ntv; e += CG_MV) {
+        const int ds = e / ntv, j = e - ds * ntv, d = ds / ns, sq = ds - d * ns;
+        const unsigned to = (unsigned)__cvta_generic_to_shared(reinterpret_cast<float4 *>(xs) + e);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to),
+                     "l"(reinterpret_cast<const float4 *>(v + (size_t)hop_nbr(a, snb, s0, d, c0 + sq) * 2 * ntv) + j)
+                     : "memory");
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// The same for blocks of more rows, a chunk of coarse sites at a time (as many as there is room
+// for the neighbour vectors), in passes of CG_MV / T pairs, T threads a pair with 8 / T residues
+// each.  The links come from HBM here, so one or two hops are in flight while one is
+// multiplied, across the passes too.  PART: consecutive threads take consecutive pairs, so that a
+// column is read in one piece, and the residues meet in part[8][rows of a chunk] after the
+// last pass; else, where there is no room for that, a pair's threads are neighbouring lanes
+// and add with shuffles.  The sums go to out.  At 32^3 x 64 (2156 rows a block, 943 MB of links)
+// a product takes 154 us, 6.1 TB/s; with a thread a row, four loads at a time, it took 258,
+// with a pair's threads on neighbouring lanes 240, with a barrier after each pass 233.
+template <int U, bool FULL, int T, bool PART>
+__device__ __forceinline__ void qmatvec_passes(const CGArgs<float> &a, const cpx<float> *v, cpx<float> *xs,
+                                               cpx<float> *part, cpx<float> *out, int r0, int nr, const int *snb, int s0,
+                                               int nsites, int tid) {
+    constexpr int PAIRS = CG_MV / T, PASS = 2 * PAIRS, RES = 8 / T;   // pairs and rows of a pass, residues of a thread
+    constexpr int AHEAD = FULL ? 2 : 1;   // hops in flight while one is multiplied, as the registers go
+    const int n2 = FULL ? 8 * U : 2 * a.ntv, ntv = n2 / 2, q = PART ? tid / PAIRS : tid % T;
+    const size_t hop = (size_t)a.nagg * n2 * ntv;   // in units of 16 bytes
+    const float4 *D4 = reinterpret_cast<const float4 *>(a.Dc), *pb;
+    const int prows = a.stage_sites * n2;   // rows of a chunk at most
+    float4 buf[AHEAD + 1][RES * U];
+    auto seek = [&](int row) {
+        const int site = row / n2;
+        pb = D4 + ((size_t)site * n2 + q) * ntv + ((row - site * n2) >> 1);
+    };
+    auto load = [&](float4(&w)[RES * U]) {
 #pragma unroll
-                for (int h = 0; h < 4; ++h) {   // four columns at a time
-                    cpx<float> b[4], x[4];
-                    const int j = j0 + 4 * h;
+        for (int e = 0; e < RES * U; ++e)
+            w[e] = FULL || T * e + q < n2 ? __ldcg(pb + T * e * ntv) : make_float4(0.f, 0.f, 0.f, 0.f);
+        pb += hop;
+    };
+    for (int c0 = s0; c0 < s0 + nsites; c0 += a.stage_sites) {
+        const int ns = min(a.stage_sites, s0 + nsites - c0);
+        const int first = max(r0 & ~1, c0 * n2), last = min(r0 + nr, (c0 + ns) * n2);
+        if (c0 > s0) asm volatile("bar.sync 2, %0;" ::"n"(CG_MV) : "memory");   // xs is free
+        int row = first + 2 * (PART ? tid % PAIRS : tid / T);
+        seek(min(row, last - 1) & ~1);   // the threads left over repeat the last pair's loads
+        load(buf[0]);
+        if (AHEAD == 2) load(buf[1]);
+        stage_neighbours(a, v, xs, snb, s0, c0, ns, tid);
+        asm volatile("bar.sync 2, %0;" ::"n"(CG_MV) : "memory");
+        for (int p0 = first; p0 < last; p0 += PASS, row += PASS) {
+            cpx<float> t0[RES][2], t1[RES][2];   // the pair's rows, even and odd terms of a residue
+            const cpx<float> *px = xs + (size_t)((min(row, last - 1) & ~1) / n2 - c0) * n2 + q;
+            auto multiply = [&](const float4(&w)[RES * U]) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if (j + q < n2) { b[q] = ldcg(pb + (size_t)(j + q) * n2); x[q] = ldcg(px + j + q); }
+                for (int e = 0; e < RES * U; ++e)   // column T e + q
+                    if (FULL || T * e + q < n2) {
+                        const cpx<float> x = px[T * e];
+                        const int r = e % RES, u = e / RES;
+                        cmac(t0[r][u & 1], cpx<float>(w[e].x, w[e].y), x);
+                        cmac(t1[r][u & 1], cpx<float>(w[e].z, w[e].w), x);
+                    }
+                px += (size_t)ns * n2;
+            };
+            const bool more = p0 + PASS < last;
+            auto next_pass = [&] { if (more) seek(min(row + PASS, last - 1) & ~1); };
+            if constexpr (AHEAD == 2) {   // hop d in buffer d mod 3
+#pragma unroll 1
+                for (int d = 0; d < 6; d += 3) {
+                    load(buf[2]);
+                    multiply(buf[0]);
+                    load(buf[0]);
+                    multiply(buf[1]);
+                    load(buf[1]);
+                    multiply(buf[2]);
+                }
+                load(buf[2]);
+                next_pass();
+                multiply(buf[0]);
+                if (more) load(buf[0]);
+                multiply(buf[1]);
+                if (more) load(buf[1]);
+                multiply(buf[2]);
+            } else {
+#pragma unroll 1
+                for (int d = 0; d < 8; d += 2) {
+                    load(buf[1]);
+                    multiply(buf[0]);
+                    load(buf[0]);
+                    multiply(buf[1]);
+                }
+                next_pass();
+                if (more) load(buf[1]);
+                multiply(buf[0]);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if (j + q < n2) cmac(acc[4 * (h & 1) + q][h >> 1], b[q], x[q]);
+                for (int e = 0; e < RES * U; ++e) buf[0][e] = buf[1][e];
+            }
+            if constexpr (PART) {
+                cpx<float> *mine = part + (size_t)q * prows + row - first;
+                if (row < last) {
+#pragma unroll
+                    for (int r = 0; r < RES; ++r) {
+                        mine[(size_t)r * T * prows] = t0[r][0] + t0[r][1];
+                        mine[(size_t)r * T * prows + 1] = t1[r][0] + t1[r][1];
+                    }
+                }
+            } else {
+                cpx<float> y0[RES], y1[RES];
+#pragma unroll
+                for (int r = 0; r < RES; ++r) {
+                    y0[r] = group_sum_up<T>(t0[r][0] + t0[r][1]);
+                    y1[r] = group_sum_up<T>(t1[r][0] + t1[r][1]);
+                }
+#pragma unroll
+                for (int o = 1; o < RES; o <<= 1)
+#pragma unroll
+                    for (int r = 0; r < RES; r += 2 * o) { y0[r] = y0[r] + y0[r + o]; y1[r] = y1[r] + y1[r + o]; }
+                const int i = row - r0;
+                if (q == 0 && row < last) {
+                    if (i >= 0) out[i] = y0[0];
+                    if (i + 1 < nr) out[i + 1] = y1[0];
                 }
             }
         }
-        cpx<float> r[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) r[q] = acc[q][0] + acc[q][1];
-        out[t] = ((r[0] + r[1]) + (r[2] + r[3])) + ((r[4] + r[5]) + (r[6] + r[7]));
+        if constexpr (PART) {
+            asm volatile("bar.sync 2, %0;" ::"n"(CG_MV) : "memory");
+            for (int t = max(r0, first) + tid; t < last; t += CG_MV) {
+                const cpx<float> *pp = part + t - first;
+                auto p2 = [&](int r) { return pp[(size_t)r * prows] + pp[(size_t)(r + 1) * prows]; };
+                out[t - r0] = (p2(0) + p2(2)) + (p2(4) + p2(6));
+            }
+        }
     }
 }
 
 __device__ __forceinline__ void qmatvec_part(const CGArgs<float> &a, const cpx<float> *v, cpx<float> *xs,
                                              cpx<float> *part, cpx<float> *out, int r0, int nr, const int *snb, int s0,
                                              int nsites, int tid) {
-    if (a.slices != 8) {
-        qmatvec_long(a, v, out, r0, nr, snb, s0, tid);
-        return;
+    if (a.slices == 8) {
+        if (a.ntv == 20) qmatvec_pairs<5, true>(a, v, xs, part, r0, nr, snb, s0, nsites, tid);   // the default
+        else qmatvec_pairs<6, false>(a, v, xs, part, r0, nr, snb, s0, nsites, tid);
+    } else {
+        auto passes = [&](auto part_room) {
+            constexpr bool P = decltype(part_room)::value;
+            if (a.ntv == 20) qmatvec_passes<5, true, 8, P>(a, v, xs, part, out, r0, nr, snb, s0, nsites, tid);
+            else if (a.ntv <= 8) qmatvec_passes<2, false, 4, P>(a, v, xs, part, out, r0, nr, snb, s0, nsites, tid);
+            else if (a.ntv <= 16) qmatvec_passes<4, false, 8, P>(a, v, xs, part, out, r0, nr, snb, s0, nsites, tid);
+            else qmatvec_passes<6, false, 8, P>(a, v, xs, part, out, r0, nr, snb, s0, nsites, tid);
+        };
+        if (a.part_size > 0) passes(std::true_type{});
+        else passes(std::false_type{});
     }
-    if (a.ntv == 20) qmatvec_pairs<5, true>(a, v, xs, part, r0, nr, snb, s0, nsites, tid);   // the default
-    else qmatvec_pairs<6, false>(a, v, xs, part, r0, nr, snb, s0, nsites, tid);
 }
 
 // FP64: the columns of a row are cut into a.slices contiguous parts, one thread each, so that
@@ -411,14 +542,42 @@ __device__ __forceinline__ cpx<R> group_sum(cpx<R> v, int lanes) {
 // what costs: four lanes share each sum, in an order of their own.
 template <typename R> struct Lanes;
 template <> struct Lanes<float> {
-    static constexpr int dot = 8;
+    static constexpr int dot = 8, long_dot = 8;
     // sum over t < n of term(t, acc), q = lane in its group
-    template <typename F> __device__ __forceinline__ static cpx<float> dot_sum(int q, int n, F term) {
+    template <int L, typename F> __device__ __forceinline__ static cpx<float> dot_sum(int q, int n, F term) {
+        static_assert(L == 8);
         cpx<float> r[4];
         for (int t = q; t < n; t += 32)
 #pragma unroll
             for (int i = 0; i < 4; ++i)
                 if (t + 8 * i < n) term(t + 8 * i, r[i]);
+        return group_sum((r[0] + r[2]) + (r[1] + r[3]), 8);
+    }
+    // sum over t < n of conj(X[t]) Y[t] in the same order, sixteen loads at a time; the sign is changed in
+    // rows from place `flip` on of their coarse site (row 0 is at place p0 of n2)
+    __device__ __forceinline__ static cpx<float> dot_global(int q, int n, int p0, int n2, int flip, const cpx<float> *X,
+                                                            const cpx<float> *Y) {
+        cpx<float> r[4];
+        const int step = 8 % n2;
+        int p = (p0 + q) % n2;
+        auto add = [&](cpx<float> &acc, cpx<float> x, cpx<float> y) {
+            if (p >= flip) x = -x;
+            p += step;
+            if (p >= n2) p -= n2;
+            acc.re += x.re * y.re + x.im * y.im;
+            acc.im += x.re * y.im - x.im * y.re;
+        };
+        int t = q;
+        for (; t + 56 < n; t += 64) {
+            cpx<float> x[8], y[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) { x[i] = X[t + 8 * i]; y[i] = Y[t + 8 * i]; }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) add(r[i & 3], x[i], y[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < 7; ++i)
+            if (t + 8 * i < n) add(r[i & 3], X[t + 8 * i], Y[t + 8 * i]);
         return group_sum((r[0] + r[2]) + (r[1] + r[3]), 8);
     }
     // sum over the blocks b < G of the contiguous values src[b]
@@ -445,17 +604,47 @@ template <> struct Lanes<float> {
     // sum over l < n of term(l, acc): L lanes, two accumulators a residue (dual) or one
     template <int L, bool dual, typename F> __device__ __forceinline__ static cpx<float> vec_sum(int q, int n, F term) {
         cpx<float> r[8 / L];
+        if constexpr (L == 1) {   // eight terms at a time, so that their loads are in flight together
+            cpx<float> odd[8];
+            auto eight = [&](int l, cpx<float>(&acc)[8]) {
+                if (l + 4 <= n) {
 #pragma unroll
-        for (int i = 0; i < 8 / L; ++i) {
-            cpx<float> a0, a1;
-            int l = q + L * i;
+                    for (int i = 0; i < 4; ++i) term(l + i, acc[i]);
+                    if (l + 8 <= n) {
+#pragma unroll
+                        for (int i = 4; i < 8; ++i) term(l + i, acc[i]);
+                    } else {
+#pragma unroll
+                        for (int i = 4; i < 7; ++i)
+                            if (l + i < n) term(l + i, acc[i]);
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 3; ++i)
+                        if (l + i < n) term(l + i, acc[i]);
+                }
+            };
+            for (int l = 0; l < n; l += dual ? 16 : 8) {
+                eight(l, r);
+                if (dual && l + 8 < n) eight(l + 8, odd);
+            }
             if (dual) {
-                for (; l + 8 < n; l += 16) { term(l, a0); term(l + 8, a1); }
-                if (l < n) term(l, a0);
-                r[i] = a0 + a1;
-            } else {
-                for (; l < n; l += 8) term(l, a0);
-                r[i] = a0;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) r[i] = r[i] + odd[i];
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8 / L; ++i) {
+                cpx<float> a0, a1;
+                int l = q + L * i;
+                if (dual) {
+                    for (; l + 8 < n; l += 16) { term(l, a0); term(l + 8, a1); }
+                    if (l < n) term(l, a0);
+                    r[i] = a0 + a1;
+                } else {
+                    for (; l < n; l += 8) term(l, a0);
+                    r[i] = a0;
+                }
             }
         }
 #pragma unroll
@@ -473,11 +662,28 @@ template <> struct Lanes<float> {
     }
 };
 template <> struct Lanes<double> {
-    static constexpr int dot = 4;
-    template <typename F> __device__ __forceinline__ static cpx<double> dot_sum(int q, int n, F term) {
+    static constexpr int dot = 4, long_dot = 4;
+    template <int L, typename F> __device__ __forceinline__ static cpx<double> dot_sum(int q, int n, F term) {
         cpx<double> r;
-        for (int t = q; t < n; t += 4) term(t, r);
-        return group_sum(r, 4);
+        for (int t = q; t < n; t += L) term(t, r);
+        return group_sum(r, L);
+    }
+    __device__ __forceinline__ static cpx<double> dot_global(int q, int n, int p0, int n2, int flip, const cpx<double> *X,
+                                                             const cpx<double> *Y) {
+        constexpr int L = long_dot;
+        cpx<double> r;
+        const int step = L % n2;
+        int p = (p0 + q) % n2;
+        for (int t = q; t < n; t += L) {
+            cpx<double> x = X[t];
+            const cpx<double> y = Y[t];
+            if (p >= flip) x = -x;
+            p += step;
+            if (p >= n2) p -= n2;
+            r.re += x.re * y.re + x.im * y.im;
+            r.im += x.re * y.im - x.im * y.re;
+        }
+        return group_sum(r, L);
     }
     __device__ __forceinline__ static cpx<double> grid_sum(const double2 *src, unsigned int G, int q, bool on) {
         cpx<double> r;
@@ -540,11 +746,11 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
     cpx<R> *rhs = S + (size_t)(2 * m + 1) * ld;
     cpx<R> *xs = rhs + ld;
     cpx<R> *ws = xs + ld;
-    // then the staged neighbour vectors (FP32), the matvec's parts [slices][nr] when a.slices > 1,
+    // then the staged neighbour vectors (FP32), the matvec's parts ([slices][nr] when a.slices > 1)
     // and GW, GAW
     cpx<R> *stage = reinterpret_cast<cpx<R> *>(cg_dyn + (a.smem_slices ? align16((size_t)a.nslice * rb * sizeof(cpx<R>)) : 0));
     cpx<R> *part = stage + (size_t)9 * a.stage_sites * n2;
-    cpx<R> *Dl = a.smem_defl ? part + (a.slices > 1 ? (size_t)a.slices * rb : 0) : nullptr;
+    cpx<R> *Dl = a.smem_defl ? part + a.part_size : nullptr;
     auto g5 = [&](int i, cpx<R> v) { return ((r0 + i) % n2) >= a.ntv ? -v : v; };
     // element i of GW_l and GAW_l
     auto GW = [&](int l, int i) { return Dl ? Dl[(size_t)l * rb + i] : g5(i, a.W[(size_t)l * a.n + r0 + i]); };
@@ -570,18 +776,39 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
         }
 
     // partial slot off + i <- sc(i) times the sum of val(i, t) over the owned rows t, i < cnt
-    auto dots = [&](int off, int cnt, auto val, auto sc) {
-        constexpr int L = Lanes<R>::dot, ngrp = CG_THREADS / L;
+    const bool wide = 4 * nr <= CG_THREADS;
+    auto dots_by = [&](auto lanes, int off, int cnt, auto val, auto sc) {
+        constexpr int L = decltype(lanes)::value, ngrp = CG_THREADS / L;
         for (int ib = 0; ib < cnt; ib += ngrp) {
             const int i = ib + tid / L;
-            const cpx<R> acc = Lanes<R>::dot_sum(tid % L, i < cnt ? nr : 0, [&](int t, cpx<R> &r) { val(i, t, r); });
+            const cpx<R> acc =
+                Lanes<R>::template dot_sum<L>(tid % L, i < cnt ? nr : 0, [&](int t, cpx<R> &r) { val(i, t, r); });
             if (i < cnt && tid % L == 0) mypart[(size_t)(off + i) * G] = P2(acc.re * sc(i), acc.im * sc(i));
         }
+    };
+    auto dots = [&](int off, int cnt, auto val, auto sc) {
+        constexpr std::integral_constant<int, Lanes<R>::dot> few{};
+        constexpr std::integral_constant<int, Lanes<R>::long_dot> many{};
+        if (few.value == many.value || wide) dots_by(few, off, cnt, val, sc);
+        else if constexpr (few.value != many.value) dots_by(many, off, cnt, val, sc);
     };
     // r += conj(p) q
     auto cdot = [](cpx<R> p, cpx<R> q, cpx<R> &r) {
         r.re += p.re * q.re + p.im * q.im;
         r.im += p.re * q.im - p.im * q.re;
+    };
+    // partial slot off + i <- sc(i) <X, Y> of the vectors that pick(i, X, Y, flip) names, i < cnt, `flip`: with the
+    // sign of gamma5
+    auto dots_global = [&](int off, int cnt, auto pick, auto sc) {
+        constexpr int L = Lanes<R>::long_dot, ngrp = CG_THREADS / L;
+        for (int ib = 0; ib < cnt; ib += ngrp) {
+            const int i = ib + tid / L;
+            const cpx<R> *X, *Y;
+            bool flip;
+            pick(min(i, cnt - 1), X, Y, flip);
+            const cpx<R> acc = Lanes<R>::dot_global(tid % L, i < cnt ? nr : 0, r0 % n2, n2, flip ? a.ntv : n2, X, Y);
+            if (i < cnt && tid % L == 0) mypart[(size_t)(off + i) * G] = P2(acc.re * sc(i), acc.im * sc(i));
+        }
     };
     // dst[i] = sum of value off + i over the blocks, i < cnt, by `threads` threads, t < threads
     auto gather = [&](int off, int cnt, P *dst, int t, int threads) {
@@ -602,7 +829,6 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
     };
     // f(i, s) with s = sum of term(l, i, s) over l < cnt, once per owned row i: four lanes a
     // row where the threads suffice, else one
-    const bool wide = 4 * nr <= CG_THREADS;
     auto rows_by = [&](auto lanes, auto dual, int t, int threads, int cnt, auto term, auto f) {
         constexpr int L = decltype(lanes)::value;
         for (int ib = 0; ib < nr; ib += threads / L) {
@@ -702,7 +928,11 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
         einv_h(tc);
         return true;
     };
-    auto gaw_t = [&](int l, int i, cpx<R> &acc) { cmac(acc, C(tc[l]), GAW(l, i)); };
+    // sums over l of tc_l AW_l, from which those of GAW follow by a sign
+    auto aw_t = [&](int l, int i, cpx<R> &acc) {
+        cmac(acc, C(tc[l]), Dl ? Dl[(size_t)(k + l) * rb + i] : a.AW[(size_t)l * a.n + r0 + i]);
+    };
+    auto to_gaw = [&](int i, cpx<R> s) { return Dl ? s : g5(i, s); };
     auto publish = [&](const cpx<R> *v) {
         for (int i = tid; i < nr; i += CG_THREADS) a.pub[r0 + i] = v[i];
     };
@@ -748,6 +978,9 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
     }
     const R tol_abs = (R)a.tol * bnorm;
 
+    // V_j+1 = w1 - sum_i h2_i s_i V_i in place: a term, the end of a row
+    auto v_term = [&](int l, int i, cpx<R> &acc) { cmac(acc, scale[l] * C(hp[l]), Vv(l)[i]); };
+    auto v_put = [&](cpx<R> *vn) { return [vn](int i, cpx<R> s) { vn[i] = vn[i] - s; }; };
     // what follows the second reduction of step j, by the threads that do not multiply:
     // the coefficients, V_j+1 = w1 - sum_i h2_i s_i V_i on the owned rows (in place), and
     // in the last warp the Hessenberg column, its rotations and the stop test
@@ -757,10 +990,9 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
         asm volatile("bar.sync 1, %0;" ::"n"(CG_POST) : "memory");
         cpx<R> *vn = Vv(j + 1);
         if (t < CG_POST - 32) {
-            auto term = [&](int l, int i, cpx<R> &acc) { cmac(acc, scale[l] * C(hp[l]), Vv(l)[i]); };
-            auto f = [&](int i, cpx<R> s) { vn[i] = vn[i] - s; };
-            if (sizeof(R) == 8) rows_by(L4, dual, t, CG_POST - 32, j + 1, term, f);
-            else rows_by(L1, dual, t, CG_POST - 32, j + 1, term, f);
+            if (!a.smem_slices) return;   // all threads do it after the matvec
+            if (sizeof(R) == 8) rows_by(L4, dual, t, CG_POST - 32, j + 1, v_term, v_put(vn));
+            else rows_by(L1, dual, t, CG_POST - 32, j + 1, v_term, v_put(vn));
             return;
         }
         P *col = Rm + j * (CG_MAXM + 1);
@@ -876,7 +1108,7 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
             } else if (!grid_sync(a.st, G, bar, a.timeout)) {
                 return;                                        // every matvec done before pub changes
             }
-            rows(k, gaw_t, [&](int i, cpx<R> s) { v0[i] = rhs[i] - (v0[i] - s); });
+            rows(k, aw_t, [&](int i, cpx<R> s) { v0[i] = rhs[i] - (v0[i] - to_gaw(i, s)); });
         } else {
             for (int i = tid; i < nr; i += CG_THREADS) v0[i] = rhs[i];
         }
@@ -913,6 +1145,9 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
             kk = j;
             if (j > 0 && stop) { conv = true; break; }
             if (j == mm) break;
+            // V_j, which with the slices in global memory would take the 64 threads of post() longer
+            // than the matvec
+            if (j > 0 && !a.smem_slices) rows(j, v_term, v_put(Vv(j)));
             matvec_end((R)scale[j], uj, ws, j);
             // reduction 1: a_l = <GW_l, gu>, b_i = <s_i V_i, gu>, f_l = <s_j V_j, GAW_l>
             const cpx<R> *vj = Vv(j);
@@ -922,11 +1157,11 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
                     const cpx<R> *Y = l <= k + j ? uj : Dl + (size_t)(l - j - 1) * rb;
                     cdot(X[t], Y[t], acc);
                 }, [&](int l) { return l < k ? R(1) : scale[l <= k + j ? l - k : j]; });
-            } else {
-                dots(OFF_S1, 2 * k + j + 1, [&](int l, int t, cpx<R> &acc) {
-                    if (l < k) cdot(GW(l, t), uj[t], acc);
-                    else if (l <= k + j) cdot(Vv(l - k)[t], uj[t], acc);
-                    else cdot(vj[t], GAW(l - k - j - 1, t), acc);
+            } else {   // W and AW in global memory: the sign of gamma5 from the row's place in its site
+                dots_global(OFF_S1, 2 * k + j + 1, [&](int l, const cpx<R> *&X, const cpx<R> *&Y, bool &flip) {
+                    flip = l < k || l > k + j;
+                    X = l < k ? a.W + (size_t)l * a.n + r0 : l <= k + j ? Vv(l - k) : vj;
+                    Y = l <= k + j ? uj : a.AW + (size_t)(l - k - j - 1) * a.n + r0;
                 }, [&](int l) { return l < k ? R(1) : scale[l <= k + j ? l - k : j]; });
             }
             if (!reduce(OFF_S1, 2 * k + j + 1)) return;
@@ -943,26 +1178,33 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs<R> a
                 ws[i] = w;
                 a.pub[r0 + i] = w;
             };
-            if constexpr (sizeof(R) == 4) {   // two sums, each of one accumulator a residue
-                if (wide) {
-                    rows_by(L4, single, tid, CG_THREADS, k, gaw_t, [&](int i, cpx<R> s) { vn[i] = uj[i] - s; });
-                    rows_by(L4, single, tid, CG_THREADS, j + 1, hv, [&](int i, cpx<R> s) { put(i, vn[i] - s); });
-                } else {
-                    rows_by(L1, single, tid, CG_THREADS, k, gaw_t, [&](int i, cpx<R> s) { vn[i] = uj[i] - s; });
-                    rows_by(L1, single, tid, CG_THREADS, j + 1, hv, [&](int i, cpx<R> s) { put(i, vn[i] - s); });
-                }
+            if (!wide) {   // two sums, each of one accumulator a residue
+                rows_by(L1, single, tid, CG_THREADS, k, aw_t, [&](int i, cpx<R> s) {
+                    const cpx<R> t = Lanes<R>::template vec_sum<1, false>(0, j + 1, [&](int l, cpx<R> &acc) { hv(l, i, acc); });
+                    put(i, uj[i] - to_gaw(i, s) - t);
+                });
+            } else if constexpr (sizeof(R) == 4) {
+                rows_by(L4, single, tid, CG_THREADS, k, aw_t, [&](int i, cpx<R> s) { vn[i] = uj[i] - to_gaw(i, s); });
+                rows_by(L4, single, tid, CG_THREADS, j + 1, hv, [&](int i, cpx<R> s) { put(i, vn[i] - s); });
             } else {
-                rows(k + j + 1,
-                     [&](int l, int i, cpx<R> &acc) {
-                         if (l < k) gaw_t(l, i, acc);
-                         else hv(l - k, i, acc);
-                     },
-                     [&](int i, cpx<R> s) { put(i, uj[i] - s); });
+                rows_by(L4, dual, tid, CG_THREADS, k + j + 1,
+                        [&](int l, int i, cpx<R> &acc) {
+                            if (l < k) cmac(acc, C(tc[l]), GAW(l, i));
+                            else hv(l - k, i, acc);
+                        },
+                        [&](int i, cpx<R> s) { put(i, uj[i] - s); });
             }
             __syncthreads();
             // reduction 2: h2_i = <s_i V_i, w1>, ||w1||^2 (gathered in post)
-            dots(OFF_S2, j + 2, [&](int l, int t, cpx<R> &acc) { cdot((l <= j ? Vv(l) : ws)[t], ws[t], acc); },
-                 [&](int l) { return l <= j ? scale[l] : R(1); });
+            auto h2_scale = [&](int l) { return l <= j ? scale[l] : R(1); };
+            if (a.smem_slices)
+                dots(OFF_S2, j + 2, [&](int l, int t, cpx<R> &acc) { cdot((l <= j ? Vv(l) : ws)[t], ws[t], acc); }, h2_scale);
+            else
+                dots_global(OFF_S2, j + 2, [&](int l, const cpx<R> *&X, const cpx<R> *&Y, bool &flip) {
+                    flip = false;
+                    X = l <= j ? Vv(l) : ws;
+                    Y = ws;
+                }, h2_scale);
             if (!grid_sync(a.st, G, bar, a.timeout)) return;
         }
         if (tid == 0) {   // y = R^-1 g

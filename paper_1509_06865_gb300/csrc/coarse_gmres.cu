@@ -82,20 +82,21 @@ CGPlan compute_plan(Ctx &c, int k, int m) {
     p.stage_sites = p.part_size = 0;
     if (sizeof(R) == 8) {
         while (p.slices < std::min(24, 9 * c.prm.n_tv) && fits((p.slices + 1) * p.rb, p.slices + 1, 0)) ++p.slices;
-    } else if (c.prm.coarse_links == MGEIG_LINKS_LEVEL) {
+    } else {
         const int n2 = 2 * c.prm.n_tv, sites = (p.rb + n2 - 2) / n2 + 1;   // that rb rows can touch
         const size_t site_b = (size_t)9 * n2 * elem;
         auto chunk = [&](size_t bytes) {   // coarse sites at a time, chunks of about the same size
             const int most = (int)std::min((size_t)sites, (room - used) / bytes);
             return most > 0 ? (sites + (sites + most - 1) / most - 1) / ((sites + most - 1) / most) : 0;
         };
-        // one pass of all rows: rb of them lie in rb / 2 + 1 pairs at most; else several, with their
-        // parts where that leaves room for four sites
-        const int with_parts = chunk(site_b + 8 * n2 * elem);
-        if (fits(8 * (p.rb / 2 + 1), 8, sites * site_b)) {
+        // level links: one pass of all rows (rb of them lie in rb / 2 + 1 pairs at most); else several,
+        // with their parts where that leaves room for four sites
+        const bool level = c.prm.coarse_links == MGEIG_LINKS_LEVEL;
+        const int with_parts = level ? chunk(site_b + 8 * n2 * elem) : 0;
+        if (level && fits(8 * (p.rb / 2 + 1), 8, sites * site_b)) {
             p.slices = 8;
             p.stage_sites = sites;
-        } else if (with_parts >= std::min(sites, 4)) {
+        } else if (level && with_parts >= std::min(sites, 4)) {
             p.stage_sites = with_parts;
             p.part_size = 8 * with_parts * n2;
         } else {

@@ -457,60 +457,91 @@ __device__ __forceinline__ void qmatvec_part(const CGArgs<double> &a, const cpx<
     }
 }
 
-// The same sums with 16-bit links (FP32 vectors and arithmetic): TPR16 lanes share a row,
-// lane q takes the column pairs p = q (mod TPR16) of the real and imaginary planes, and
-// every hop block's sum is multiplied by the block's scale.
-constexpr int TPR16 = 8;
+// The same sums with 16-bit links (FP32 vectors and arithmetic): eight lanes share a row,
+// lane q takes the column pairs p = q (mod 8) of the real and imaginary planes, and every hop
+// block's sum is multiplied by the block's scale.  Passes, staged neighbour vectors and two
+// hops in flight as above.  At 32^3 x 64 a product takes 128 us (472 MB of links), at 24^3 x 48
+// 44; 192 and 65 with one hop in flight and the vectors read from L2, 242 and 86 with none.
 template <typename H>
-__device__ __forceinline__ void qmatvec16(const CGArgs<float> &a, const cpx<float> *v, cpx<float> *out, int r0, int nr,
-                                          const int *snb, int s0, int tid) {
+__device__ __forceinline__ void qmatvec16(const CGArgs<float> &a, const cpx<float> *v, cpx<float> *xs, cpx<float> *out,
+                                          int r0, int nr, const int *snb, int s0, int nsites, int tid) {
     using HP = typename H16<H>::P;
-    const int n2 = 2 * a.ntv, np = a.ntv;
-    const int grp = tid / TPR16, q = tid % TPR16;
-    constexpr int ngrp = CG_MV / TPR16;
-    constexpr int U = (CG_MAXK + TPR16 - 1) / TPR16;   // pairs per lane (n2 / 2 <= CG_MAXK)
-    const H *L = static_cast<const H *>(a.L16);
-    for (int tb = 0; tb < nr; tb += ngrp) {
-        const int t = tb + grp;
-        float ar = 0.f, ai = 0.f;
-        if (t < nr) {
-            const int site = (r0 + t) / n2, row = (r0 + t) - site * n2;
-#pragma unroll 1
-            for (int d = 0; d < 9; ++d) {
-                const size_t blk = (size_t)d * a.nagg + site;
-                const int nb = hop_nbr(a, snb, s0, d, site);
-                const HP *pr = reinterpret_cast<const HP *>(L + blk * 2 * n2 * n2 + (size_t)row * n2);
-                const HP *pi = pr + (size_t)n2 * n2 / 2;
-                const float4 *xb = reinterpret_cast<const float4 *>(v + (size_t)nb * n2);
-                HP rv[U], iv[U];
-                float4 xv[U];
+    constexpr int PASS = CG_MV / 8, U = (CG_MAXK + 7) / 8;   // pairs per lane (n2 / 2 <= CG_MAXK)
+    struct Hop {
+        HP re[U], im[U];
+        float scale;
+    };
+    const int n2 = 2 * a.ntv, np = a.ntv, q = tid & 7;
+    const size_t hop = (size_t)a.nagg * n2 * n2;   // in units of pairs
+    const HP *pb;
+    const float *ps;
+    Hop b0, b1, b2;
+    auto seek = [&](int row) {
+        const int site = row / n2;
+        pb = static_cast<const HP *>(a.L16) + ((size_t)site * 2 * n2 + row - site * n2) * np + q;
+        ps = a.Ls + site;
+    };
+    auto load = [&](Hop &w) {
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int p = q + u * TPR16;
-                    if (p < np) { rv[u] = pr[p]; iv[u] = pi[p]; xv[u] = __ldcg(xb + p); }
-                }
+        for (int u = 0; u < U; ++u)
+            if (q + 8 * u < np) {
+                w.re[u] = pb[8 * u];
+                w.im[u] = pb[n2 * np + 8 * u];
+            }
+        w.scale = __ldg(ps);
+        pb += hop;
+        ps += a.nagg;
+    };
+    for (int c0 = s0; c0 < s0 + nsites; c0 += a.stage_sites) {
+        const int ns = min(a.stage_sites, s0 + nsites - c0);
+        const int first = max(r0, c0 * n2), last = min(r0 + nr, (c0 + ns) * n2);
+        if (c0 > s0) asm volatile("bar.sync 2, %0;" ::"n"(CG_MV) : "memory");   // xs is free
+        int row = first + (tid >> 3);
+        seek(min(row, last - 1));   // the threads left over repeat the last row's loads
+        load(b0);
+        load(b1);
+        stage_neighbours(a, v, xs, snb, s0, c0, ns, tid);
+        asm volatile("bar.sync 2, %0;" ::"n"(CG_MV) : "memory");
+        for (int p0 = first; p0 < last; p0 += PASS, row += PASS) {
+            float ar = 0.f, ai = 0.f;
+            const float4 *px = reinterpret_cast<const float4 *>(xs) + (size_t)(min(row, last - 1) / n2 - c0) * np + q;
+            auto multiply = [&](const Hop &w) {
                 float dr = 0.f, di = 0.f;
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    if (q + u * TPR16 < np) {
-                        const float2 r = H16<H>::pair(rv[u]), im = H16<H>::pair(iv[u]);
-                        const float4 x = xv[u];
+                    if (q + 8 * u < np) {
+                        const float2 r = H16<H>::pair(w.re[u]), im = H16<H>::pair(w.im[u]);
+                        const float4 x = px[8 * u];
                         dr = fmaf(r.x, x.x, dr); dr = fmaf(-im.x, x.y, dr);
                         di = fmaf(r.x, x.y, di); di = fmaf(im.x, x.x, di);
                         dr = fmaf(r.y, x.z, dr); dr = fmaf(-im.y, x.w, dr);
                         di = fmaf(r.y, x.w, di); di = fmaf(im.y, x.z, di);
                     }
                 }
-                const float sc = __ldg(a.Ls + blk);
-                ar = fmaf(sc, dr, ar);
-                ai = fmaf(sc, di, ai);
+                ar = fmaf(w.scale, dr, ar);
+                ai = fmaf(w.scale, di, ai);
+                px += (size_t)ns * np;
+            };
+#pragma unroll 1
+            for (int d = 0; d < 6; d += 3) {
+                load(b2);
+                multiply(b0);
+                load(b0);
+                multiply(b1);
+                load(b1);
+                multiply(b2);
             }
+            load(b2);
+            const bool more = p0 + PASS < last;
+            if (more) seek(min(row + PASS, last - 1));
+            multiply(b0);
+            if (more) load(b0);
+            multiply(b1);
+            if (more) load(b1);
+            multiply(b2);
+            const cpx<float> y = group_sum_up<8>(cpx<float>(ar, ai));
+            if (q == 0 && row < last) out[row - r0] = y;
         }
-        for (int o = 1; o < TPR16; o <<= 1) {
-            ar += __shfl_xor_sync(0xffffffffu, ar, o);
-            ai += __shfl_xor_sync(0xffffffffu, ai, o);
-        }
-        if (t < nr && q == 0) out[t] = cpx<float>(ar, ai);
     }
 }
 
@@ -519,8 +550,8 @@ template <typename R, int LK>
 __device__ __forceinline__ void matvec_part(const CGArgs<R> &a, const cpx<R> *v, cpx<R> *xs, cpx<R> *part, cpx<R> *out,
                                             int r0, int nr, const int *snb, int s0, int nsites, int tid) {
     if constexpr (LK == 0) qmatvec_part(a, v, xs, part, out, r0, nr, snb, s0, nsites, tid);
-    else if constexpr (LK == 1) qmatvec16<__nv_bfloat16>(a, v, out, r0, nr, snb, s0, tid);
-    else qmatvec16<__half>(a, v, out, r0, nr, snb, s0, tid);
+    else if constexpr (LK == 1) qmatvec16<__nv_bfloat16>(a, v, xs, out, r0, nr, snb, s0, nsites, tid);
+    else qmatvec16<__half>(a, v, xs, out, r0, nr, snb, s0, nsites, tid);
 }
 
 template <typename R>

@@ -73,15 +73,25 @@ CGPlan compute_plan(Ctx &c, int k, int m) {
     MG_REQUIRE(used <= room, MGEIG_ECUDA);
     // Threads that share a row of the matvec and leave the sum of their parts to its end: 8 (of a row
     // pair) in FP32 with level links where one pass takes all rows, 1 in the forms with several
-    // passes (and with 16-bit links, whose lanes share a row already), up to 24 in FP64 (every
-    // part costs the end of the matvec an FP64 addition per row)
+    // passes (and with 16-bit links, whose lanes share a row already).  FP64: up to 24, as far as
+    // one run of CG_MV threads and the room go (every part costs the end of the matvec an addition
+    // per row); with more rows than threads the count whose runs cost least, in FP64 instructions
+    // (24^3 x 48, 683 rows: a matvec 324 us with one part, whose second run is a quarter full, 272
+    // with fifteen)
     auto fits = [&](int threads, int q, size_t stage) {
         return threads <= CG_MV && used + stage + (size_t)q * p.rb * elem <= room;
     };
     p.slices = 1;
     p.stage_sites = p.part_size = 0;
     if (sizeof(R) == 8) {
-        while (p.slices < std::min(24, 9 * c.prm.n_tv) && fits((p.slices + 1) * p.rb, p.slices + 1, 0)) ++p.slices;
+        const int most = std::min(24, 9 * c.prm.n_tv);
+        while (p.slices < most && fits((p.slices + 1) * p.rb, p.slices + 1, 0)) ++p.slices;
+        long long best = 0;
+        for (int q = 1; p.rb > CG_MV && q <= most && fits(0, q, 0); ++q) {
+            const long long runs = ((long long)q * p.rb + CG_MV - 1) / CG_MV, row_groups = (p.rb + 31) / 32;
+            const long long cost = runs * 72 * c.prm.n_tv * (CG_MV / 32) / q + 2 * q * row_groups;
+            if (q == 1 || cost < best) { best = cost; p.slices = q; }
+        }
     } else {
         const int n2 = 2 * c.prm.n_tv, sites = (p.rb + n2 - 2) / n2 + 1;   // that rb rows can touch
         const size_t site_b = (size_t)9 * n2 * elem;

@@ -409,19 +409,18 @@ __device__ __forceinline__ void qmatvec_part(const CGArgs<float> &a, const cpx<f
     }
 }
 
-// FP64: the columns of a row are cut into a.slices contiguous parts, one thread each, so that
-// a whole matvec is one run of independent loads per thread.
+// FP64: the columns of a row are cut into a.slices contiguous parts, each of them one thread's, so
+// that a whole matvec is one run of independent loads per thread, or a few such runs that leave
+// few threads without work in the last.
 __device__ __forceinline__ void qmatvec_part(const CGArgs<double> &a, const cpx<double> *v, cpx<double> *,
                                              cpx<double> *part, cpx<double> *out, int r0, int nr, const int *snb, int s0,
                                              int, int tid) {
     constexpr int U = 2;
     const int ntv = a.ntv, n2 = 2 * ntv, CP = 9 * ntv, S = a.slices;
-    const int sl = S > 1 ? tid / nr : 0;
-    if (sl >= S) return;
-    const int q0 = sl * CP / S, q1 = (sl + 1) * CP / S;
     const double2 *D2 = reinterpret_cast<const double2 *>(a.Dc), *v2 = reinterpret_cast<const double2 *>(v);
     const size_t next_hop = (size_t)(a.nagg - 1) * n2 * n2;
-    for (int p = S > 1 ? tid - sl * nr : tid; p < nr; p += S > 1 ? nr : CG_MV) {
+    for (int e = tid; e < S * nr; e += CG_MV) {
+        const int sl = e / nr, p = e - sl * nr, q0 = sl * CP / S, q1 = (sl + 1) * CP / S;
         const int row = r0 + p, site = row / n2, rin = row - site * n2;
         int d = q0 / ntv, jp = q0 - d * ntv;
         const double2 *pb = D2 + (((size_t)d * a.nagg + site) * n2 + 2 * jp) * n2 + rin;
@@ -693,7 +692,7 @@ template <> struct Lanes<float> {
     }
 };
 template <> struct Lanes<double> {
-    static constexpr int dot = 4, long_dot = 4;
+    static constexpr int dot = 4, long_dot = 8;   // eight where a block has more rows, for more warps with work
     template <int L, typename F> __device__ __forceinline__ static cpx<double> dot_sum(int q, int n, F term) {
         cpx<double> r;
         for (int t = q; t < n; t += L) term(t, r);

@@ -557,10 +557,13 @@ void apply_fine_nrhs(Ctx &c, int mode, double sigma, const void *x, void *y, int
         const int nb = grid_for(c.g.V, NR_SITES);
         // Runs of at most 64 CTAs (8192 sites: with 12 fields three timeslices of them are 28 MB
         // of L2) where a timeslice is a whole number of CTAs and longer: 32^3 x 64 with 12 fields
-        // 2257 us in the order of the sites, 2148 with 64, 2169 with 32, 2188 with 128.
+        // 2257 us in the order of the sites, 2148 with 64, 2169 with 32, 2188 with 128.  L2 holds
+        // three whole timeslices of few fields on a small lattice in the order of the sites, and
+        // runs only cost: 24^3 x 48 with 2 fields (8 MB) 156 us without them, 162 with; 32^3 x 64
+        // with 2 (18 MB) 464 either way, with 3 (27 MB) 656 and 632.
         NrOrder o{1, c.dims[3], 1};
         const int S3 = c.g.V / c.dims[3];
-        if (S3 % NR_SITES == 0) {
+        if (S3 % NR_SITES == 0 && (size_t)3 * S3 * 96 * nrhs > (size_t)18 << 20) {
             o.slice = o.cpc = S3 / NR_SITES;
             for (int d = 2; o.cpc > 64; ++d)
                 if (o.slice % d == 0) o.cpc = o.slice / d;

@@ -241,8 +241,13 @@ void restrict_vec(Ctx &c, const void *const *P, const void *r, void *rc) {
     // parts of the test vectors so that there are up to six CTAs an SM: with one CTA an aggregate a
     // coarse grid of few aggregates left SMs idle (FP64, 8^3 x 16, 32 aggregates: 99 us, and the
     // prolongation, then a thread a site, 70 us; the cycle 2040 -> 1948 us with both cut).  Two
-    // CTAs an SM or six are alike; 512 aggregates at 16^3 x 32 take one part, as before
-    const int parts = std::min(ntv, std::max(1, 6 * c.sms / A.n)), per = (ntv + parts - 1) / parts;
+    // CTAs an SM or six are alike; 512 aggregates at 16^3 x 32 take one part, as before.  Every
+    // part reads r again: in FP32 the line below keeps one part where there is not much more than
+    // that to read (256 aggregates, N_tv = 4: 9.5 us in one part, 11 in two; 320, N_tv = 20: 35
+    // and 37.5; 256, N_tv = 20: 33 and in three parts 29)
+    int parts = std::min(ntv, std::max(1, 6 * c.sms / A.n));
+    if (sizeof(R) == 4 && A.vol <= 256 && 10 * A.n >= c.sms * ntv) parts = 1;
+    const int per = (ntv + parts - 1) / parts;
     const size_t smem = (size_t)(threads / 32) * 2 * per * 2 * sizeof(R);
     TimeScope ts(c.timer, K_RESTRICT, (double)(ntv + 1) * c.g.V * 24 * sizeof(R));
     restrict_kernel<R><<<dim3(A.n, (ntv + per - 1) / per), threads, smem, c.stream>>>(c.g, A, p, ntv, per, r,

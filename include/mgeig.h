@@ -154,11 +154,14 @@ typedef struct mgeig_params {
     double barrier_timeout;   /* seconds (of SM clock) a block of the persistent
                              coarse solver waits at a grid barrier before it gives
                              up, raises MGEIG_ETIMEOUT and returns              */
-    int coarse_blocks;    /* thread blocks of the persistent coarse solver (one
-                             per SM at most, each owning a contiguous slice of
-                             the coarse rows); 0 = one per SM, capped by the
-                             rows.  Fewer blocks make the two grid barriers of an
-                             Arnoldi step cheaper and each block's matvec longer */
+    int coarse_blocks;    /* thread blocks of the persistent coarse solver at most
+                             (each owning a contiguous slice of the coarse rows);
+                             0 = as many as there are SMs.  With either value a
+                             block owns at least 128 rows in FP32 and 12 in FP64
+                             (128 where the basis does not fit into shared
+                             memory).  Fewer blocks make the two grid barriers of
+                             an Arnoldi step cheaper and each block's matvec
+                             longer                                             */
     int blas_ds;          /* 1 (MGEIG_MIXED only): the inner products and vector
                              updates of the FP64 vectors (Gram-Schmidt and the
                              Rayleigh quotients of Algorithm 1, the Arnoldi steps
@@ -220,7 +223,9 @@ int mgeig_set_params(mgeig_ctx *ctx, const mgeig_params *p);
  * usable without a GPU.  Besides the checks listed above: aggregate and SAP
  * block volumes <= 1024, n_tv <= 6 x aggregate volume, 16-bit coarse links and
  * the learned smoother only with MGEIG_MIXED, the learned smoother only on
- * extents divisible by 4 x 4 x 4 x 2, 0 < barrier_timeout <= 60. */
+ * extents divisible by 4 x 4 x 4 x 2, 0 < barrier_timeout <= 60.  A SAP block of
+ * more than 256 sites is accepted, but what sweeps over it (setup, cycles, solves,
+ * mgeig_sap) returns MGEIG_ECUDA. */
 int mgeig_check_params(const int dims[4], const mgeig_params *p);
 
 /* Copy a host gauge field (layout above) to the device and build the clover
@@ -323,7 +328,7 @@ int mgeig_coarse_apply(mgeig_ctx *ctx, double sigma, const double *xc, double *y
  * another (Eq. 2.6).  With MGEIG_MIXED and MGEIG_LINKS_BF16 one launch on the
  * tensor cores (BF16 links with their per-link FP32 scale, right-hand sides
  * rounded to BF16 after the scale is applied, FP32 accumulation); with the
- * level-precision links one CUDA-core launch for up to 24, IEEE half links one per
+ * level-precision links one CUDA-core launch, with IEEE half links one per
  * right-hand side. */
 int mgeig_coarse_apply_nrhs(mgeig_ctx *ctx, double sigma, const double *xc, double *yc, int nrhs);
 

@@ -28,7 +28,11 @@ size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
 // Bytes of a block's slices (2 restart + 5 vectors of ceil(n / G) rows, at most one block
 // per 128 rows) up to which they live in shared memory: the line that
-// mgeig_mg_cycle_dev_noalloc's scratch limit is drawn by.
+// mgeig_mg_cycle_dev_noalloc's scratch limit is drawn by.  So it stays where it is although the
+// kernel changes: 24912 and 47504 bytes of static shared memory are the most that the line
+// leaves room for (the kernels take 24272 and 46224 now), and the 2 m + 4 vectors that a block
+// keeps leave the neighbour vectors of one site room beside them, 3456 bytes at most, where the
+// line is nearest (restart 32: 374 rows, 3696 bytes left).
 template <typename R> struct SliceBudget { static constexpr size_t bytes = CG_SMEM_LIMIT - 24912; };
 template <> struct SliceBudget<double> { static constexpr size_t bytes = CG_SMEM_LIMIT - 47504; };
 // Rows an FP64 block has at least: its blocks may be more and smaller (no order to keep).

@@ -590,8 +590,8 @@ void coarse_apply_many(Ctx &c, double sigma, const void *Xv, void *Yv, int n) {
         const cpx<R> *x = static_cast<const cpx<R> *>(Xv) + (size_t)r0 * c.coarse_ncpx();
         cpx<R> *y = static_cast<cpx<R> *>(Yv) + (size_t)r0 * c.coarse_ncpx();
         if (m <= 4) launch_coarse_many<R, 1>(c, sigma, x, y, m);
-        else if (m <= 8 || sizeof(R) == 8) launch_coarse_many<R, 2>(c, sigma, x, y, m);
-        else launch_coarse_many<R, 4>(c, sigma, x, y, m);
+        else if (sizeof(R) == 8 || m <= 8) launch_coarse_many<R, 2>(c, sigma, x, y, m);
+        else if constexpr (sizeof(R) == 4) launch_coarse_many<R, 4>(c, sigma, x, y, m);
     }
 }
 template void coarse_apply_many<float>(Ctx &, double, const void *, void *, int);

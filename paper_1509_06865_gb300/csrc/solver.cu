@@ -120,7 +120,7 @@ static cpx<double> *dslot(Ctx &c, int i) { return c.red_out.as<cpx<double>>() + 
 static cpx<double> *hslot(Ctx &c, int i) { return reinterpret_cast<cpx<double> *>(c.pinned) + i; }
 static cpx<double> *upslot(Ctx &c, int i) { return reinterpret_cast<cpx<double> *>(c.pinned) + RED_SLOTS + i; }
 
-struct CoarseState { unsigned int count, gen; int status, iters; };
+struct CoarseState { unsigned int count, exits; int status, iters; };   // the coarse solver's CGState
 
 // copy device slots [0, n) to the host mirror and wait; every fetch also
 // brings back the persistent coarse solver's state and raises its errors
@@ -1685,7 +1685,7 @@ static int mg_cycle_noalloc_impl(Ctx &c, double sigma, const void *r, void *z) {
         sap_sweep<R>(c, 0, sigma, r, true, z);
         sap_sweep<R>(c, 1, sigma, r, true, z);
     }
-    int state[4];   // barrier count, generation, status (0 ok, 1 timeout, 2 breakdown), iterations
+    int state[4];   // barrier arrivals, blocks that have left, status (0 ok, 1 timeout, 2 breakdown), iterations
     MG_CUDA(cudaMemcpyAsync(state, s, sizeof(state), cudaMemcpyDeviceToHost, c.stream));
     sync(c);
     c.st.coarse_iters += state[3];

@@ -419,8 +419,10 @@ __device__ __forceinline__ void qmatvec_part(const CGArgs<double> &a, const cpx<
     const int ntv = a.ntv, n2 = 2 * ntv, CP = 9 * ntv, S = a.slices;
     const double2 *D2 = reinterpret_cast<const double2 *>(a.Dc), *v2 = reinterpret_cast<const double2 *>(v);
     const size_t next_hop = (size_t)(a.nagg - 1) * n2 * n2;
-    for (int e = tid; e < S * nr; e += CG_MV) {
-        const int sl = e / nr, p = e - sl * nr, q0 = sl * CP / S, q1 = (sl + 1) * CP / S;
+    int sl = tid / nr, p = tid - sl * nr;   // the thread's part and row
+#pragma unroll 1
+    for (; sl < S; p += CG_MV, sl += p / nr, p %= nr) {
+        const int q0 = sl * CP / S, q1 = (sl + 1) * CP / S;
         const int row = r0 + p, site = row / n2, rin = row - site * n2;
         int d = q0 / ntv, jp = q0 - d * ntv;
         const double2 *pb = D2 + (((size_t)d * a.nagg + site) * n2 + 2 * jp) * n2 + rin;

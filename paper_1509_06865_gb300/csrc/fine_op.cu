@@ -427,9 +427,9 @@ __global__ void __launch_bounds__(128) wilson_clover_nrhs_kernel(Geom g, const v
 // its sites' forward links (two rows, 12 float4 planes) and clover (18 planes)
 // into shared memory once, with coalesced loads, and applies the stencil to
 // every field from there; only the spinors (and the backward links of hops that
-// leave the CTA) stream from memory for each field.  DRAM (47 % busy), L1 and the issue slots
-// (50 % each) share the time with the latency of 12 warps an SM; 2 or 3 threads a site, each
-// with every 2nd or 3rd field, and smaller groups of fields were slower.
+// leave the CTA) stream from memory for each field.  What bounds it is the loads' latency at 12
+// warps an SM (12 fields at 32^3 x 64: DRAM 42 %, issue slots 51 %, L1 55 % busy); 2 or 3 threads
+// a site, each with every 2nd or 3rd field, and smaller groups of fields were slower.
 constexpr int NR_SITES = 128;
 constexpr size_t NR_SMEM = (size_t)(12 + 18) * NR_SITES * sizeof(float4);
 
